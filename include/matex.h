@@ -133,16 +133,14 @@ typedef struct matex_opts {
                               of the rounds in one launch when they fit a quarter of the free
                               memory; 3: as 2, but each round kernel solves its own (the path
                               taken when they do not fit; the same results bit for bit) */
-  int32_t tc_solve;        /* supernodes at least tc_min_width wide in the level solves: 0
-                              (default) chosen at setup per column count, 1 off, 2 on.  Their
-                              two dense products per supernode (P_s b_s forward, P_s^T [..]
-                              backward) run on the bf16 tensor cores as an error-free split of
-                              the FP64 operands into nine 6-bit digits (error of the order of an
-                              FP64 dot product), the rest of each level on the FP64 kernels.
-                              With 0 the setup times the solve pair both ways at each column
-                              count it tunes and keeps the tensor cores where they are faster.
-                              Level launches only (not the persistent solve) */
-  int32_t tc_min_width;    /* 0 (default): 64; else at least 32 */
+  int32_t tc_solve;        /* the level solves' dense products (P_s b_s forward, P_s^T [..]
+                              backward) on the tensor cores: 0 (default) for two columns and
+                              more, and for one where the setup times it faster; 1 off; 2 for
+                              every column count.  An error-free split of the FP64 operands into
+                              seven 8-bit digits (error no larger than an FP64 dot product's),
+                              one launch per tree level and direction (solve_mode 1 and 2) */
+  int32_t tc_min_width;    /* 0 (default): 64; else at least 32: the width from which
+                              tc_solve_supernodes counts */
   int32_t single_column;   /* solves of one right-hand side: 0 (default) chosen at setup, 1 off,
                               2 on.  The single-column level kernels run one launch per tree level
                               and direction like the level launches, with everything that does
@@ -184,8 +182,8 @@ typedef struct matex_stats {
                               window tape and reverse work buffers (tape 2) */
   int32_t tc_rounds;       /* segment rounds of the last run whose V y ran on the tensor cores */
   int32_t resident;        /* 1: the segment rounds run as resident rounds (opts.resident) */
-  int32_t tc_solve_supernodes;  /* supernodes whose solve products can run on the tensor cores
-                                   (0: none or tc_solve off) */
+  int32_t tc_solve_supernodes;  /* supernodes at least tc_min_width wide whose solve products
+                                   can run on the tensor cores (0: none or tc_solve off) */
   int32_t tc_solve_min_cols;    /* smallest column count at which they do (0: never) */
   int32_t single_column;        /* 1: single-column solves run the single-column level kernels */
 } matex_stats;
@@ -471,6 +469,22 @@ matex_status matex_host_factor_solve(int64_t n, const int64_t* rowptr, const int
                                      const double* val, const double* dshift, double alpha,
                                      int32_t max_width, int32_t ncols, const double* b, double* x,
                                      int64_t* info);
+
+/*
+ * Host-only check of the work plan of the tensor-core level solves (the
+ * operator apply of Alg. 1 and the input solves of Eq. 5/6), no GPU needed:
+ * factors diag(dshift) + alpha A as matex_host_factor_solve does, builds the
+ * plan of matex_setup, and solves for ncols right-hand sides in FP64 by walking
+ * the plan's tasks as the kernels do (version 0: wide tasks, 1: narrow ones;
+ * cluster 1 to 8: thread blocks sharing a long reduction).  Every panel tile
+ * must be taken exactly once or hold zeros.  info (host [4], may be NULL)
+ * receives {supernodes, tasks of both directions, those with several chunks,
+ * mapping errors}; MATEX_ERR_STATE when there is one.
+ */
+matex_status matex_host_tensor_plan(int64_t n, const int64_t* rowptr, const int32_t* col,
+                                    const double* val, const double* dshift, double alpha,
+                                    int32_t max_width, int32_t version, int32_t cluster,
+                                    int32_t ncols, const double* b, double* x, int64_t* info);
 
 /*
  * Host-only check of the work plan of the single-column level kernels (the

@@ -87,23 +87,49 @@ bool partial_ldlt(double* F, int64_t nr, int64_t w, double* dinv, std::vector<do
 
 }  // namespace
 
+// Column k of the panel [L_ss^{-1}; L_Rs L_ss^{-1}] of the supernode at
+// columns j0 .. j0 + w of the front (leading dimension nr), whose rows below
+// are the front's rows at[0 .. r): x[0 .. w) by forward substitution on e_k,
+// x[w .. w + r) = L_Rs x[0 .. w).  at = null: the rows right below the columns.
+void panel_column(const double* front, int64_t nr, int64_t j0, int64_t w, int64_t r,
+                  const int32_t* at, int64_t k, double* x) {
+  x[k] = 1.0;
+  for (int64_t j = k; j < w; ++j) {
+    const double xj = x[j];
+    if (xj == 0.0) continue;
+    const double* cj = &front[(j0 + j) * nr];
+    for (int64_t i = j + 1; i < w; ++i) x[i] -= cj[j0 + i] * xj;
+    if (at)
+      for (int64_t i = 0; i < r; ++i) x[w + i] += cj[at[i]] * xj;
+    else
+      for (int64_t i = 0; i < r; ++i) x[w + i] += cj[j0 + w + i] * xj;
+  }
+}
+
 std::string numeric_ldlt(const CsrSym& A, const double* dshift, double alpha,
-                         const Symbolic& S, Numeric& F) {
+                         const Symbolic& S, Numeric& F, const Symbolic* coarse,
+                         std::vector<double>* coarse_pan) {
+  // the elimination runs on the coarse structure when there is one (larger
+  // fronts, fewer extend-adds); S's panels are cut from its columns of L
+  const Symbolic& T = coarse ? *coarse : S;
   const int64_t n = S.n;
   F.dinv.assign(n, 0.0);
   F.pan_cm.assign(S.pan_off[S.nsup], 0.0);
   F.pan_rm.assign(S.pan_off[S.nsup], 0.0);
+  if (coarse_pan) coarse_pan->assign(T.pan_off[T.nsup], 0.0);
   std::vector<int32_t> pos(n, -1);
-  std::vector<std::vector<double>> upd(S.nsup);
-  std::vector<std::vector<int32_t>> kids(S.nsup);
-  for (int32_t s = 0; s < S.nsup; ++s)
-    if (S.sup_parent[s] >= 0) kids[S.sup_parent[s]].push_back(s);
+  std::vector<std::vector<double>> upd(T.nsup);
+  std::vector<std::vector<int32_t>> kids(T.nsup);
+  for (int32_t s = 0; s < T.nsup; ++s)
+    if (T.sup_parent[s] >= 0) kids[T.sup_parent[s]].push_back(s);
   std::vector<double> front, lcol;
-  for (int32_t s = 0; s < S.nsup; ++s) {
-    const int32_t f = S.sup_first[s], l = S.sup_first[s + 1];
+  std::vector<int32_t> at;
+  int32_t fs = 0;  // first supernode of S in the front
+  for (int32_t s = 0; s < T.nsup; ++s) {
+    const int32_t f = T.sup_first[s], l = T.sup_first[s + 1];
     const int64_t w = l - f;
-    const int32_t* R = &S.sup_rows[S.sup_rowptr[s]];
-    const int64_t nr = S.sup_rowptr[s + 1] - S.sup_rowptr[s];
+    const int32_t* R = &T.sup_rows[T.sup_rowptr[s]];
+    const int64_t nr = T.sup_rowptr[s + 1] - T.sup_rowptr[s];
     const int64_t r = nr - w;
     for (int64_t k = 0; k < nr; ++k) pos[R[k]] = (int32_t)k;
     front.assign(nr * nr, 0.0);
@@ -121,9 +147,9 @@ std::string numeric_ldlt(const CsrSym& A, const double* dshift, double alpha,
     }
     // extend-add the children's update matrices
     for (int32_t c : kids[s]) {
-      const int64_t wc = S.sup_first[c + 1] - S.sup_first[c];
-      const int32_t* Rc = &S.sup_rows[S.sup_rowptr[c] + wc];
-      const int64_t rc = S.sup_rowptr[c + 1] - S.sup_rowptr[c] - wc;
+      const int64_t wc = T.sup_first[c + 1] - T.sup_first[c];
+      const int32_t* Rc = &T.sup_rows[T.sup_rowptr[c] + wc];
+      const int64_t rc = T.sup_rowptr[c + 1] - T.sup_rowptr[c] - wc;
       const std::vector<double>& U = upd[c];
       std::vector<int32_t> rel(rc);
       for (int64_t a = 0; a < rc; ++a) rel[a] = pos[Rc[a]];
@@ -137,31 +163,34 @@ std::string numeric_ldlt(const CsrSym& A, const double* dshift, double alpha,
     // partial factorisation of the first w columns
     if (!partial_ldlt(front.data(), nr, w, &F.dinv[f], lcol))
       return "matrix is not symmetric positive definite";
-    // solve panel P = [L_ss^{-1}; L_Rs L_ss^{-1}]: column k of L_ss^{-1} by
-    // forward substitution on e_k, then column k of L_Rs L_ss^{-1}
-    double* pcm = &F.pan_cm[S.pan_off[s]];
-    double* prm = &F.pan_rm[S.pan_off[s]];
-    const int64_t ld = w + r;
-    const double pwork = (double)w * (double)w * (double)ld / 2.0;
-    parallel_for(w, pwork, [&](int64_t lo, int64_t hi) {
-      for (int64_t k = lo; k < hi; ++k) {
-        double* x = &pcm[k * ld];  // x[0..w) = L_ss^{-1} e_k, x[w..w+r) = L_Rs x[0..w)
-        x[k] = 1.0;
-        for (int64_t j = k; j < w; ++j) {
-          const double xj = x[j];
-          if (xj == 0.0) continue;
-          const double* cj = &front[j * nr];
-          for (int64_t i = j + 1; i < w; ++i) x[i] -= cj[i] * xj;
-          for (int64_t i = 0; i < r; ++i) x[w + i] += cj[w + i] * xj;
-        }
-      }
-    });
-    parallel_for(ld, (double)w * ld, [&](int64_t lo, int64_t hi) {
-      for (int64_t i = lo; i < hi; ++i)
-        for (int64_t k = 0; k < w; ++k) prm[i * w + k] = pcm[k * ld + i];
-    });
+    // solve panels of S's supernodes in this front
+    for (; fs < S.nsup && S.sup_first[fs] < l; ++fs) {
+      const int64_t j0 = S.sup_first[fs] - f, wf = S.sup_first[fs + 1] - S.sup_first[fs];
+      const int64_t ld = S.sup_rowptr[fs + 1] - S.sup_rowptr[fs], rf = ld - wf;
+      const int32_t* Rf = &S.sup_rows[S.sup_rowptr[fs] + wf];
+      at.resize(rf);
+      for (int64_t i = 0; i < rf; ++i) at[i] = pos[Rf[i]];
+      const int32_t* rows = coarse ? at.data() : nullptr;
+      double* pcm = &F.pan_cm[S.pan_off[fs]];
+      double* prm = &F.pan_rm[S.pan_off[fs]];
+      parallel_for(wf, (double)wf * (double)wf * (double)ld / 2.0, [&](int64_t lo, int64_t hi) {
+        for (int64_t k = lo; k < hi; ++k)
+          panel_column(front.data(), nr, j0, wf, rf, rows, k, &pcm[k * ld]);
+      });
+      parallel_for(ld, (double)wf * ld, [&](int64_t lo, int64_t hi) {
+        for (int64_t i = lo; i < hi; ++i)
+          for (int64_t k = 0; k < wf; ++k) prm[i * wf + k] = pcm[k * ld + i];
+      });
+    }
+    if (coarse_pan) {
+      double* pan = &(*coarse_pan)[T.pan_off[s]];
+      parallel_for(w, (double)w * (double)w * (double)nr / 2.0, [&](int64_t lo, int64_t hi) {
+        for (int64_t k = lo; k < hi; ++k)
+          panel_column(front.data(), nr, 0, w, r, nullptr, k, &pan[k * nr]);
+      });
+    }
     // Schur complement handed to the parent
-    if (r > 0 && S.sup_parent[s] >= 0) {
+    if (r > 0 && T.sup_parent[s] >= 0) {
       std::vector<double>& U = upd[s];
       U.assign(r * r, 0.0);
       for (int64_t b = 0; b < r; ++b)

@@ -151,6 +151,174 @@ void nd_rec(NdState& st, std::vector<int32_t>& nodes) {
   st.out->insert(st.out->end(), S.begin(), S.end());
 }
 
+// The supernodes that amalgamation left (gone: merged into another), renumbered.
+void keep_supernodes(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
+                     std::vector<int32_t>& col2sup, std::vector<int64_t>& zeros,
+                     const std::vector<int32_t>& first, const std::vector<char>& gone) {
+  std::vector<int32_t> keep;
+  for (int32_t t = 0; t < (int32_t)gone.size(); ++t)
+    if (!gone[t]) keep.push_back(t);
+  std::sort(keep.begin(), keep.end(), [&](int32_t a, int32_t b) { return first[a] < first[b]; });
+  std::vector<std::vector<int32_t>> rows2(keep.size());
+  std::vector<int64_t> zeros2(keep.size());
+  S.sup_first.assign(keep.size() + 1, 0);
+  for (size_t k = 0; k < keep.size(); ++k) {
+    S.sup_first[k] = first[keep[k]];
+    rows2[k].swap(offrows[keep[k]]);
+    zeros2[k] = zeros[keep[k]];
+  }
+  zeros.swap(zeros2);
+  S.nsup = (int32_t)keep.size();
+  S.sup_first[S.nsup] = (int32_t)S.n;
+  for (int32_t t = 0; t < S.nsup; ++t)
+    for (int32_t j = S.sup_first[t]; j < S.sup_first[t + 1]; ++j) col2sup[j] = t;
+  S.sup_parent.assign(S.nsup, -1);
+  for (int32_t t = 0; t < S.nsup; ++t)
+    if (!rows2[t].empty()) S.sup_parent[t] = col2sup[rows2[t][0]];
+  offrows.swap(rows2);
+}
+
+// Supernodes renumbered, every parent's children with the largest subtree
+// first: the small ones end up adjacent to their parent.  Only the numbering
+// changes, no panel.
+void order_children(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
+                    std::vector<int32_t>& col2sup, std::vector<int64_t>& zeros) {
+  const int32_t ns = S.nsup;
+  std::vector<int64_t> size(ns);
+  std::vector<std::vector<int32_t>> kids(ns);
+  std::vector<int32_t> stack, order;
+  for (int32_t s = 0; s < ns; ++s) size[s] += S.sup_first[s + 1] - S.sup_first[s];
+  for (int32_t s = 0; s < ns; ++s)
+    if (S.sup_parent[s] >= 0) {  // children come before their parent
+      size[S.sup_parent[s]] += size[s];
+      kids[S.sup_parent[s]].push_back(s);
+    }
+  for (int32_t r = ns - 1; r >= 0; --r)
+    if (S.sup_parent[r] < 0) stack.push_back(r);
+  // parents before children, the largest subtree last; then backwards
+  while (!stack.empty()) {
+    const int32_t s = stack.back();
+    stack.pop_back();
+    order.push_back(s);
+    std::stable_sort(kids[s].begin(), kids[s].end(),
+                     [&](int32_t a, int32_t b) { return size[a] > size[b]; });
+    stack.insert(stack.end(), kids[s].begin(), kids[s].end());
+  }
+  std::reverse(order.begin(), order.end());
+  std::vector<int32_t> first(ns + 1, 0), map(S.n), pos(ns), perm(S.n), par(ns);
+  std::vector<std::vector<int32_t>> rows(ns);
+  std::vector<int64_t> z(ns);
+  for (int32_t k = 0; k < ns; ++k) {
+    const int32_t s = order[k], w = S.sup_first[s + 1] - S.sup_first[s];
+    pos[s] = k;
+    first[k + 1] = first[k] + w;
+    z[k] = zeros[s];
+    for (int32_t j = 0; j < w; ++j) {
+      map[S.sup_first[s] + j] = first[k] + j;
+      perm[first[k] + j] = S.perm[S.sup_first[s] + j];
+      col2sup[first[k] + j] = k;
+    }
+  }
+  for (int32_t s = 0; s < ns; ++s) {
+    par[pos[s]] = S.sup_parent[s] < 0 ? -1 : pos[S.sup_parent[s]];
+    std::vector<int32_t>& r = rows[pos[s]];
+    r.swap(offrows[s]);
+    for (int32_t& i : r) i = map[i];
+    std::sort(r.begin(), r.end());
+  }
+  S.sup_first.swap(first);
+  S.sup_parent.swap(par);
+  S.perm.swap(perm);
+  for (int64_t k = 0; k < S.n; ++k) S.iperm[S.perm[k]] = (int32_t)k;
+  offrows.swap(rows);
+  zeros.swap(z);
+}
+
+// Amalgamation for the tensor-core solves (k_sptrsv_mma.cu), whose unit of
+// work is a 16 x 16 block of the panel, on top of the relaxed one: a child
+// adjacent to its parent joins it when the merged panel costs no more than the
+// two: blocks, plus kRow per panel row (splitting or conversion and atomics of
+// its right-hand sides), plus kSup per supernode (a thread block's chain of
+// loads).  On the 180k-node grid 4,350 supernodes in 15 levels come from 27,600
+// in 18, the blocks grow by a tenth, the panel rows shrink from 683k to 425k;
+// kSup of 0.5 to 8 and kRow of 0.05 to 0.2 measured within 5 %, a limit of 0.6
+// on the zeros 12 % slower than 0.8.
+void amalgamate_tiled(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
+                      std::vector<int32_t>& col2sup, std::vector<int64_t>& zeros, int32_t max_width) {
+  constexpr double kRow = 0.12, kSup = 2.0, kMaxZeros = 0.8;
+  const int32_t ns = S.nsup;
+  std::vector<int32_t> first(S.sup_first.begin(), S.sup_first.end() - 1);
+  std::vector<int32_t> last(S.sup_first.begin() + 1, S.sup_first.end());
+  std::vector<char> gone(ns, 0);
+  std::vector<std::vector<int32_t>> kids(ns);
+  for (int32_t t = 0; t < ns; ++t)
+    if (S.sup_parent[t] >= 0) kids[S.sup_parent[t]].push_back(t);
+  auto cost = [&](int64_t w, int64_t ld) {
+    return (double)((w + 15) / 16) * (double)((ld + 15) / 16) + kRow * (double)ld + kSup;
+  };
+  for (int32_t p = 0; p < ns; ++p) {
+    std::vector<int32_t>& ch = kids[p];
+    const int64_t rp = (int64_t)offrows[p].size();
+    while (!ch.empty()) {
+      const int32_t t = ch.back();  // the child that ends where p begins
+      if (last[t] != first[p]) break;
+      const int64_t ws = last[t] - first[t], wp = last[p] - first[p], w = ws + wp;
+      const int64_t rt = (int64_t)offrows[t].size();
+      const int64_t z = zeros[t] + zeros[p] + ws * (wp + rp - rt);
+      const double dense = (double)w * (double)(w + 1) / 2.0 + (double)w * (double)rp;
+      if (w > max_width || (double)z > kMaxZeros * dense ||
+          cost(w, w + rp) > cost(ws, ws + rt) + cost(wp, wp + rp))
+        break;
+      first[p] = first[t];
+      zeros[p] = z;
+      gone[t] = 1;
+      ch.pop_back();
+      // its own children are p's now; the last of them may end where p begins
+      ch.insert(ch.end(), kids[t].begin(), kids[t].end());
+    }
+  }
+  keep_supernodes(S, offrows, col2sup, zeros, first, gone);
+}
+
+// Row lists, panel offsets and levels of the supernodes found.
+void lay_out(Symbolic& S, const std::vector<std::vector<int32_t>>& offrows) {
+  S.sup_rowptr.assign(S.nsup + 1, 0);
+  S.pan_off.assign(S.nsup + 1, 0);
+  S.nnz_L = 0;
+  S.flops_factor = 0;
+  for (int32_t s = 0; s < S.nsup; ++s) {
+    int64_t w = S.sup_first[s + 1] - S.sup_first[s];
+    int64_t r = (int64_t)offrows[s].size();
+    S.sup_rowptr[s + 1] = S.sup_rowptr[s] + w + r;
+    S.pan_off[s + 1] = S.pan_off[s] + (w + r) * w;
+    S.nnz_L += w * (w - 1) / 2 + w * r;
+    double nr = (double)(w + r);
+    S.flops_factor += (double)w * nr * nr;  // order of the partial factorisation cost
+  }
+  S.sup_rows.resize(S.sup_rowptr[S.nsup]);
+  for (int32_t s = 0; s < S.nsup; ++s) {
+    int64_t q = S.sup_rowptr[s];
+    for (int32_t j = S.sup_first[s]; j < S.sup_first[s + 1]; ++j) S.sup_rows[q++] = j;
+    for (int32_t i : offrows[s]) S.sup_rows[q++] = i;
+  }
+  // levels of the supernodal tree, leaves first
+  std::vector<int32_t> lev(S.nsup, 0);
+  int32_t maxlev = 0;
+  for (int32_t s = 0; s < S.nsup; ++s) {
+    int32_t p = S.sup_parent[s];
+    if (p >= 0) lev[p] = std::max(lev[p], lev[s] + 1);
+    maxlev = std::max(maxlev, lev[s]);
+  }
+  S.level_ptr.assign(maxlev + 2, 0);
+  for (int32_t s = 0; s < S.nsup; ++s) S.level_ptr[lev[s] + 1]++;
+  for (int32_t l = 0; l <= maxlev; ++l) S.level_ptr[l + 1] += S.level_ptr[l];
+  S.level_sups.resize(S.nsup);
+  {
+    std::vector<int32_t> fill(S.level_ptr.begin(), S.level_ptr.end() - 1);
+    for (int32_t s = 0; s < S.nsup; ++s) S.level_sups[fill[lev[s]]++] = s;
+  }
+}
+
 }  // namespace
 
 std::string nested_dissection(const CsrSym& A, std::vector<int32_t>& perm) {
@@ -171,7 +339,7 @@ std::string nested_dissection(const CsrSym& A, std::vector<int32_t>& perm) {
 }
 
 std::string symbolic_analysis(const CsrSym& A, const std::vector<int32_t>& nd_perm,
-                              int32_t max_width, Symbolic& S) {
+                              int32_t max_width, Symbolic& S, Symbolic* coarse) {
   const int64_t n = A.n;
   std::vector<int32_t> ip(n);
   for (int64_t k = 0; k < n; ++k) ip[nd_perm[k]] = (int32_t)k;
@@ -322,10 +490,11 @@ std::string symbolic_analysis(const CsrSym& A, const std::vector<int32_t>& nd_pe
   // block stay small; fewer, wider supernodes mean fewer tree levels and
   // denser panels for the solves.  Thresholds: merged width <= 4 always;
   // <= 16 with < 80% zeros; <= 48 with < 10%; otherwise < 5%.
+  std::vector<int64_t> zeros;  // explicit zeros of each supernode's panel
   {
     const int32_t ns = S.nsup;
     std::vector<int32_t> first(ns), last(ns);
-    std::vector<int64_t> zeros(ns, 0);
+    zeros.assign(ns, 0);
     std::vector<char> gone(ns, 0);
     for (int32_t t = 0; t < ns; ++t) {
       first[t] = S.sup_first[t];
@@ -347,60 +516,17 @@ std::string symbolic_analysis(const CsrSym& A, const std::vector<int32_t>& nd_pe
       zeros[par] = z;
       gone[t] = 1;
     }
-    std::vector<int32_t> keep;
-    for (int32_t t = 0; t < ns; ++t)
-      if (!gone[t]) keep.push_back(t);
-    std::sort(keep.begin(), keep.end(), [&](int32_t a, int32_t b) { return first[a] < first[b]; });
-    std::vector<std::vector<int32_t>> rows2(keep.size());
-    S.sup_first.assign(keep.size() + 1, 0);
-    for (size_t k = 0; k < keep.size(); ++k) {
-      S.sup_first[k] = first[keep[k]];
-      rows2[k].swap(offrows[keep[k]]);
-    }
-    S.nsup = (int32_t)keep.size();
-    S.sup_first[S.nsup] = (int32_t)n;
-    for (int32_t t = 0; t < S.nsup; ++t)
-      for (int32_t j = S.sup_first[t]; j < S.sup_first[t + 1]; ++j) col2sup[j] = t;
-    S.sup_parent.assign(S.nsup, -1);
-    for (int32_t t = 0; t < S.nsup; ++t)
-      if (!rows2[t].empty()) S.sup_parent[t] = col2sup[rows2[t][0]];
-    offrows.swap(rows2);
+    keep_supernodes(S, offrows, col2sup, zeros, first, gone);
   }
-  S.sup_rowptr.assign(S.nsup + 1, 0);
-  S.pan_off.assign(S.nsup + 1, 0);
-  S.nnz_L = 0;
-  S.flops_factor = 0;
-  for (int32_t s = 0; s < S.nsup; ++s) {
-    int64_t w = S.sup_first[s + 1] - S.sup_first[s];
-    int64_t r = (int64_t)offrows[s].size();
-    S.sup_rowptr[s + 1] = S.sup_rowptr[s] + w + r;
-    S.pan_off[s + 1] = S.pan_off[s] + (w + r) * w;
-    S.nnz_L += w * (w - 1) / 2 + w * r;
-    double nr = (double)(w + r);
-    S.flops_factor += (double)w * nr * nr;  // order of the partial factorisation cost
+  order_children(S, offrows, col2sup, zeros);
+  if (coarse) {
+    *coarse = S;
+    std::vector<std::vector<int32_t>> rows = offrows;
+    std::vector<int32_t> c2s = col2sup;
+    amalgamate_tiled(*coarse, rows, c2s, zeros, max_width);
+    lay_out(*coarse, rows);
   }
-  S.sup_rows.resize(S.sup_rowptr[S.nsup]);
-  for (int32_t s = 0; s < S.nsup; ++s) {
-    int64_t q = S.sup_rowptr[s];
-    for (int32_t j = S.sup_first[s]; j < S.sup_first[s + 1]; ++j) S.sup_rows[q++] = j;
-    for (int32_t i : offrows[s]) S.sup_rows[q++] = i;
-  }
-  // levels of the supernodal tree, leaves first
-  std::vector<int32_t> lev(S.nsup, 0);
-  int32_t maxlev = 0;
-  for (int32_t s = 0; s < S.nsup; ++s) {
-    int32_t p = S.sup_parent[s];
-    if (p >= 0) lev[p] = std::max(lev[p], lev[s] + 1);
-    maxlev = std::max(maxlev, lev[s]);
-  }
-  S.level_ptr.assign(maxlev + 2, 0);
-  for (int32_t s = 0; s < S.nsup; ++s) S.level_ptr[lev[s] + 1]++;
-  for (int32_t l = 0; l <= maxlev; ++l) S.level_ptr[l + 1] += S.level_ptr[l];
-  S.level_sups.resize(S.nsup);
-  {
-    std::vector<int32_t> fill(S.level_ptr.begin(), S.level_ptr.end() - 1);
-    for (int32_t s = 0; s < S.nsup; ++s) S.level_sups[fill[lev[s]]++] = s;
-  }
+  lay_out(S, offrows);
   return "";
 }
 

@@ -52,10 +52,15 @@ struct Numeric {
 // Host setup (host_symbolic.cpp / host_numeric.cpp).  Both return an empty
 // string on success, else a message.
 std::string nested_dissection(const CsrSym& A, std::vector<int32_t>& perm);
+// coarse (or null): the same columns in larger supernodes, each a run of S's,
+// for the tensor-core solves.
 std::string symbolic_analysis(const CsrSym& A, const std::vector<int32_t>& nd_perm,
-                              int32_t max_width, Symbolic& S);
-// Factor diag(dshift) + alpha*A; dshift may be null (then just alpha*A).
+                              int32_t max_width, Symbolic& S, Symbolic* coarse = nullptr);
+// Factor diag(dshift) + alpha*A; dshift may be null (then just alpha*A).  With
+// a coarse structure (symbolic_analysis), coarse_pan (or null) receives its
+// panels too, column-major.
 std::string numeric_ldlt(const CsrSym& A, const double* dshift, double alpha,
-                         const Symbolic& S, Numeric& F);
+                         const Symbolic& S, Numeric& F, const Symbolic* coarse = nullptr,
+                         std::vector<double>* coarse_pan = nullptr);
 
 }  // namespace matex

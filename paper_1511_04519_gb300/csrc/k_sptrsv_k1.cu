@@ -123,7 +123,8 @@ k1_fwd_kernel(DevFactor F, const K1Sup* __restrict__ sups, int nsup,
     else orow = __ldg(F.sup_rows + L.d.rp + i);
   }
   k1_chain_wait();
-  if (F.abort && *F.abort) return;
+  // in flight beside the right-hand side; nothing is written when it is set
+  const bool stop = F.abort && __ldcg(F.abort);
   const double* __restrict__ b = Y + (int64_t)L.d.f * ldy;
   double acc = 0.0, acc2 = 0.0;
   for (int tr = 0; tr < trips; ++tr) {
@@ -151,7 +152,7 @@ k1_fwd_kernel(DevFactor F, const K1Sup* __restrict__ sups, int nsup,
     }
   }
   acc = k1_group_sum(acc + acc2, G);
-  if (L.live && L.sub == 0) {
+  if (L.live && L.sub == 0 && !stop) {
     if (i < w) Y2[(int64_t)(L.d.f + i) * ldy] = acc * dinv;
     else atomicAdd(Y + (int64_t)orow * ldy, -acc);
   }
@@ -195,7 +196,8 @@ k1_bwd_kernel(DevFactor F, const K1Sup* __restrict__ sups, int nsup,
   for (int tp = 0; tp < kPre; ++tp)
     if (tp < trips) load_g(g[tp], tp);
   k1_chain_wait();
-  if (F.abort && *F.abort) return;
+  // in flight beside the right-hand side; nothing is written when it is set
+  const bool stop = F.abort && __ldcg(F.abort);
   const double* __restrict__ y = Y2 + (int64_t)L.d.f * ldy;
   double acc = 0.0, acc2 = 0.0;
   auto step = [&](const int (&gg)[kK1Terms], int tr) {
@@ -224,7 +226,7 @@ k1_bwd_kernel(DevFactor F, const K1Sup* __restrict__ sups, int nsup,
     step(gg, tr);
   }
   acc = k1_group_sum(acc + acc2, G);
-  if (L.live && L.sub == 0) Y[(int64_t)(L.d.f + k) * ldy] = acc;
+  if (L.live && L.sub == 0 && !stop) Y[(int64_t)(L.d.f + k) * ldy] = acc;
 }
 
 }  // namespace

@@ -1,6 +1,7 @@
 // Launch wrappers of the R-MATEX CUDA kernels (internal to the library).
 #pragma once
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
@@ -529,41 +530,58 @@ struct K1Plan {
 // chained by programmatic dependent launch; returns the launches
 int solve_k1(const DevFactor& F, const K1Plan& P, double* Y, double* Y2, int ldy, cudaStream_t st);
 
-// Wide supernodes of the level solves on the tensor cores (k_sptrsv_tc.cu).
-// Per wide supernode: its panel (offset pan, first node f, width w, rows ld,
-// row list rp), the row tiles of the forward (ld rows) and backward (w rows)
-// products, and the offsets of its panel slices (a_f, a_b: bytes into the
-// direction's slice store of the factor) and of its row scales (rs_f, rs_b,
-// in doubles).
-struct TsSup {
-  int64_t pan, rp;
-  int32_t f, w, ld, mt_f, mt_b, pad;
-  int64_t a_f, a_b, rs_f, rs_b;
+// Multi-right-hand-side level solves on the tensor cores (k_sptrsv_mma.cu).
+// Per direction and supernode: its panel (offset pan, first node f, width w,
+// rows ld), the 8-row tiles and 16-term K steps of its product (forward
+// ld x w, backward w x ld), its first tile a (row tile major) and where its
+// rows' results go (klist[8 dl..]).
+struct MmSup {
+  int64_t pan, a;
+  int32_t f, w, ld, rt, ks, dl;
 };
-// One tree level's wide supernodes (indices into the TsSup table) and the
-// tiles of its two products: {supernode, row tile | K slice << 16}.
-struct TsLevel {
-  int32_t nsup = 0, ntile_f = 0, ntile_b = 0;
-  const int32_t* list = nullptr;
-  const int2* tiles_f = nullptr;
-  const int2* tiles_b = nullptr;
+constexpr int kMmCols = 16;         // right-hand sides of a thread block
+constexpr int kMmPack = 8;          // supernodes of a packed task (their K steps fit one chunk)
+constexpr int kMmRowsWide = 32, kMmRowsNarrow = 4;  // most row tiles of a task, two versions
+// Flag in a node index: backward, read x of an ancestor from Y (without it
+// y_s from Y2); forward, subtract from an ancestor's row of Y.
+constexpr int kMmAdd = 1 << 30;
+// A task: nu units (one row tile each) from u0; K steps [kbeg, kend) whose
+// right-hand-side rows are klist[16 (kl + k)..]; the supernode (of the pack) of
+// K step k in bits 4 (k & 7).. of emap; klist[8 dl..]: where the row tiles'
+// results go (multi-chunk tasks).  A unit: {first tile of the row tile, K
+// steps kb | ke << 16, supernode | slot of its K step 0 << 16, 0}.
+struct MmTask {
+  int32_t u0, nu, kl, kbeg, kend, dl;
+  uint32_t emap, pad;
 };
-constexpr int kTsMinWidth = 64;  // default: supernodes at least this wide use the tensor cores
-size_t ts_a_bytes(int rows, int kdim);   // panel slices of one product
-int ts_row_tiles(int rows);
-int ts_k_slices(int kdim);               // CTAs sharing one row tile (split reduction)
-void ts_set_limits();
-// panel slices and row scales of nsup wide supernodes (max_mt: most row tiles)
-void ts_split_panels(const DevFactor& F, const TsSup* sups, int nsup, int max_mt, bool fwd,
-                     __nv_bfloat16* A, double* rowscale, cudaStream_t st);
-// the wide supernodes of one level, one direction, ncols right-hand sides of
-// the solve buffers (Y node-major, Y2 the forward intermediate)
-void ts_solve_level(const DevFactor& F, const TsSup* sups, const TsLevel& L, bool fwd,
-                    const __nv_bfloat16* A, const double* rowscale, double* Y, double* Y2, int ldy,
-                    int ncols, int32_t* err, cudaStream_t st);
-// one level launch of the FP64 solve (k_sptrsv.cu), the level's own tuned
-// column block
-void solve_level(bool fwd, const DevFactor& F, const LevelPlan& L, double* Y, double* Y2, int ldy,
-                 int ncols, cudaStream_t st, const SplitScratch* split);
+// One level, one direction: its tasks, those with more than one chunk (at most
+// kMmRowsNarrow row tiles) first; steps: the most K steps of any of those.
+struct MmLevel {
+  const MmTask* tasks = nullptr;
+  int32_t nmulti = 0, nsingle = 0, steps = 1;
+};
+// A level takes its wide tasks from 3 CTAs per SM on (below, narrow ones spread
+// the level further; 6 and 12 a SM measured 2 and 8 % slower at 64 columns on
+// the 180k-node grid), a cluster shares a task's K steps while that adds CTAs
+// up to 2 per SM (1: 5 % slower, 4: 4 %), at least two steps each, and the
+// ring of panel tiles is deep up to 3 CTAs per SM, all of them resident at once.
+constexpr int kMmFill = 3 * 152, kMmClusterFill = 2 * 152, kMmDeep = 3 * 152;
+struct MmPlan {
+  int32_t nlev = 0, nsup = 0;
+  const MmSup* sups[2] = {};             // per direction (0 forward), in task order
+  const int4* units[2] = {};
+  const int32_t* klist[2] = {};
+  std::vector<MmLevel> lev[2][2];        // [direction][0 wide, 1 narrow tasks]
+  unsigned char* A[2][2] = {};           // panel tiles [factor C + gamma G, G][direction]
+};
+size_t mm_tile_bytes();
+bool mm_set_limits();
+// panel tiles of one direction from the column-major panels pan (device) of a
+// factor and its D^{-1}
+void mm_split_panels(const double* pan, const double* dinv, const MmPlan& P, bool fwd,
+                     unsigned char* A, cudaStream_t st);
+// one solve pair of ncols columns (fi: 0 = C + gamma G, 1 = G); returns the launches
+int solve_mm(const int32_t* abort, const MmPlan& P, int fi, double* Y, double* Y2, int ldy, int ncols,
+             cudaStream_t st);
 
 }  // namespace matex

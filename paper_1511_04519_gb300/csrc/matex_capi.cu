@@ -78,24 +78,16 @@ struct matex_ctx {
   std::vector<double> pwl_v_host_shape;  // length of pwl_v
   // structure
   Symbolic S;
+  Symbolic SC;                     // S in larger supernodes, for the tensor-core solves
   std::vector<LevelPlan> levels;
   SplitScratch split;              // chunked reductions of the level launches
   // resident rounds (opts.resident): per-level work lists, the choice, and
   // the setup's timings of one solve pair both ways (ms, -1 if not taken)
-  // wide supernodes on the tensor cores (opts.tc_solve): the level plans
-  // without their split tasks, per level their (supernode, row tile) lists,
-  // the panel slices and row scales of both factors and directions, the
-  // and per column count whether a call uses them
-  int ts_minw = 0;
-  std::vector<LevelPlan> levels_n;
-  std::vector<TsLevel> ts_levels;
-  TsSup* ts_sups = nullptr;
-  int ts_n = 0;
-  __nv_bfloat16* tsA[2][2] = {};   // [factor M, G][forward, backward]
-  double* tsR[2][2] = {};
-  int ts_mtf = 0, ts_mtb = 0;      // most row tiles of a wide supernode, per direction
-  std::vector<int8_t> ts_by_ncols;
-  int ts_min_cols = 0;
+  // level solves on the tensor cores (opts.tc_solve, k_sptrsv_mma.cu): plan,
+  // panel digits, and per column count whether a solve takes them
+  MmPlan mm;
+  bool mm_ok = false;
+  std::vector<int8_t> mm_by_ncols;
   ResidentPlan rplan;
   ResFactor rM, rG;          // the factors' resident copies
   ResStoreSup* rsup = nullptr;
@@ -573,34 +565,6 @@ bool plan_levels(matex_ctx* c) {
     c->levels[l].ftasks = fd + fofs[l];
     c->levels[l].btasks = bd + bofs[l];
   }
-  if (c->ts_minw > 0) {
-    // the same task lists without the split tasks of supernodes at least
-    // ts_minw wide (packed tasks hold supernodes at most 16 wide)
-    std::vector<int2> ftn, btn;
-    std::vector<size_t> fon(nlev + 1), bon(nlev + 1);
-    auto narrow = [&](const int2& t) { return t.x < 0 || sup_w(t.x) < c->ts_minw; };
-    for (int l = 0; l < nlev; ++l) {
-      fon[l] = ftn.size();
-      bon[l] = btn.size();
-      for (size_t e = fofs[l]; e < fofs[l + 1]; ++e)
-        if (narrow(ft[e])) ftn.push_back(ft[e]);
-      for (size_t e = bofs[l]; e < bofs[l + 1]; ++e)
-        if (narrow(bt[e])) btn.push_back(bt[e]);
-    }
-    fon[nlev] = ftn.size();
-    bon[nlev] = btn.size();
-    int2 *fdn = nullptr, *bdn = nullptr;
-    if (!c->upload(fdn, ftn.data(), ftn.size()) || !c->upload(bdn, btn.data(), btn.size()))
-      return false;
-    c->levels_n = c->levels;
-    for (int l = 0; l < nlev; ++l) {
-      LevelPlan& L = c->levels_n[l];
-      L.ftasks = fdn + fon[l];
-      L.btasks = bdn + bon[l];
-      L.nf = (int32_t)(fon[l + 1] - fon[l]);
-      L.nb = (int32_t)(bon[l + 1] - bon[l]);
-    }
-  }
   set_solve_smem_limit(std::max(smem_need, kSolveSmemTune));
   // persistent schedules for every column count 1..ldy
   std::vector<PersistLevel> pl((size_t)c->ldy * nlev);
@@ -945,191 +909,268 @@ void autotune_k1(matex_ctx* c) {
   }
 }
 
-// Tensor-core products of the wide supernodes (k_sptrsv_tc.cu): their table,
-// per level the (supernode, row tile) lists of both directions, and the
-// panel slices of both factors.  False when there is no wide supernode or no
-// room (at most a quarter of the free memory), and the solves stay FP64.
-bool plan_ts(matex_ctx* c) {
-  const Symbolic& S = c->S;
+// Tensor-core level solves (k_sptrsv_mma.cu): per direction the supernodes by
+// level, the units and row lists, and the two versions of every level's tasks.
+struct MmHostPlan {
+  std::vector<MmSup> sups;
+  std::vector<int4> units;
+  std::vector<int32_t> klist;
+  std::vector<MmTask> tasks[2];
+  struct Range { size_t t0; int nmulti, nsingle, steps; };
+  std::vector<Range> lev[2];
+  int64_t tiles = 0;
+};
+
+void build_mm_plan(const Symbolic& S, bool fwd, MmHostPlan& P) {
+  constexpr int kCh = 8;  // K steps of a chunk
   const int nlev = (int)S.level_ptr.size() - 1;
-  // the narrow levels launch with the column blocks tuned for the full ones
-  for (int l = 0; l < nlev && l < (int)c->levels_n.size(); ++l) {
-    c->levels_n[l].kbf = c->levels[l].kbf;
-    c->levels_n[l].kbb = c->levels[l].kbb;
-  }
-  std::vector<int32_t> wid(S.nsup, -1);
-  std::vector<TsSup> sups;
-  int64_t aF = 0, aB = 0, rF = 0, rB = 0;
-  int mtf = 0, mtb = 0;
-  for (int32_t s = 0; s < S.nsup; ++s) {
-    const int f = S.sup_first[s], w = S.sup_first[s + 1] - f;
-    if (w < c->ts_minw) continue;
-    const int ld = (int)(S.sup_rowptr[s + 1] - S.sup_rowptr[s]);
-    TsSup d{};
-    d.pan = S.pan_off[s];
-    d.rp = S.sup_rowptr[s];
-    d.f = f;
-    d.w = w;
-    d.ld = ld;
-    d.mt_f = ts_row_tiles(ld);
-    d.mt_b = ts_row_tiles(w);
-    d.a_f = aF;
-    aF += (int64_t)ts_a_bytes(ld, w);
-    d.a_b = aB;
-    aB += (int64_t)ts_a_bytes(w, ld);
-    d.rs_f = rF;
-    rF += 128LL * d.mt_f;
-    d.rs_b = rB;
-    rB += 128LL * d.mt_b;
-    mtf = std::max(mtf, d.mt_f);
-    mtb = std::max(mtb, d.mt_b);
-    wid[s] = (int32_t)sups.size();
-    sups.push_back(d);
-  }
-  if (sups.empty()) return false;
-  const double need = 2.0 * (double)(aF + aB) + 16.0 * (double)(rF + rB);
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
-  if (need > 0.25 * (double)free_b) return false;
-  std::vector<int32_t> list;
-  std::vector<int2> tf, tb;
-  std::vector<size_t> lo(nlev + 1), fo(nlev + 1), bo2(nlev + 1);
   for (int l = 0; l < nlev; ++l) {
-    lo[l] = list.size();
-    fo[l] = tf.size();
-    bo2[l] = tb.size();
-    for (int k = S.level_ptr[l]; k < S.level_ptr[l + 1]; ++k) {
-      const int j = wid[S.level_sups[k]];
-      if (j < 0) continue;
-      list.push_back(j);
-      const int kf = ts_k_slices(sups[j].w), kb = ts_k_slices(sups[j].ld);
-      for (int kc = 0; kc < kf; ++kc)
-        for (int mt = 0; mt < sups[j].mt_f; ++mt) tf.push_back(make_int2(j, mt | (kc << 16)));
-      for (int kc = 0; kc < kb; ++kc)
-        for (int mt = 0; mt < sups[j].mt_b; ++mt) tb.push_back(make_int2(j, mt | (kc << 16)));
+    // the level's supernodes, longest reduction first, so that packs hold alike ones
+    std::vector<MmSup> lv;
+    std::vector<int64_t> lrow;
+    std::vector<int32_t> ids(S.level_sups.begin() + S.level_ptr[l], S.level_sups.begin() + S.level_ptr[l + 1]);
+    auto steps_rows = [&](int32_t s) {
+      const int w = S.sup_first[s + 1] - S.sup_first[s], ld = (int)(S.sup_rowptr[s + 1] - S.sup_rowptr[s]);
+      return fwd ? std::make_pair((w + 15) / 16, ld) : std::make_pair((ld + 15) / 16, w);
+    };
+    std::stable_sort(ids.begin(), ids.end(), [&](int32_t x, int32_t y) { return steps_rows(x) > steps_rows(y); });
+    for (const int32_t s : ids) {
+      lrow.push_back(S.sup_rowptr[s]);
+      MmSup d{};
+      d.pan = S.pan_off[s];
+      d.f = S.sup_first[s];
+      d.w = S.sup_first[s + 1] - d.f;
+      d.ld = (int32_t)(S.sup_rowptr[s + 1] - S.sup_rowptr[s]);
+      d.rt = ((fwd ? d.ld : d.w) + 7) / 8;
+      d.ks = ((fwd ? d.w : d.ld) + 15) / 16;
+      lv.push_back(d);
+    }
+    // right-hand-side rows of every K step and result rows of every row tile
+    std::vector<int32_t> kl, dl;
+    for (size_t i = 0; i < lv.size(); ++i) {
+      MmSup& d = lv[i];
+      const int32_t* rows = &S.sup_rows[lrow[i]];
+      d.a = P.tiles;
+      P.tiles += (int64_t)d.rt * d.ks;
+      kl.push_back((int32_t)(P.klist.size() / 16));
+      for (int k = 0; k < d.ks * 16; ++k)
+        P.klist.push_back(k >= (fwd ? d.w : d.ld) ? -1
+                          : k < d.w ? d.f + k : rows[k] | kMmAdd);
+      d.dl = (int32_t)(P.klist.size() / 8);
+      dl.push_back(d.dl);
+      for (int r = 0; r < (d.rt + 1) / 2 * 16; ++r)
+        P.klist.push_back(r >= (fwd ? d.ld : d.w) ? -1
+                          : r < d.w ? d.f + r : rows[r] | kMmAdd);
+      P.sups.push_back(d);
+    }
+    for (int ver = 0; ver < 2; ++ver) {
+      const int R = ver == 0 ? kMmRowsWide : kMmRowsNarrow;
+      struct T { MmTask t; int chunks; long long cost; };
+      std::vector<T> multi, single;
+      // K steps of row tile rt: the triangle of L_ss^{-1} ends the forward's
+      // rows inside the diagonal block and starts the backward's
+      auto steps = [&](const MmSup& d, int rt, int& kb, int& ke) {
+        kb = fwd ? 0 : rt / 2;
+        ke = fwd && (rt + 1) * 8 <= d.w ? std::min(d.ks, rt / 2 + 1) : d.ks;
+      };
+      auto unit = [&](const MmSup& d, int rt, int e, int slot) {
+        int kb, ke;
+        steps(d, rt, kb, ke);
+        P.units.push_back(make_int4((int)(d.a + (int64_t)rt * d.ks), kb | (ke << 16), e | (slot << 16), 0));
+        return ke - kb;
+      };
+      for (size_t i = 0; i < lv.size();) {
+        const MmSup& d = lv[i];
+        if (d.ks > kCh || d.rt > R) {
+          const int r = d.ks > kCh ? kMmRowsNarrow : R;
+          const int nblk = (d.rt + r - 1) / r;
+          for (int b = 0; b < nblk; ++b) {
+            const int r0 = d.rt * b / nblk, r1 = d.rt * (b + 1) / nblk;
+            T t{};
+            t.t.u0 = (int32_t)P.units.size();
+            t.t.nu = r1 - r0;
+            t.t.kl = kl[i];
+            t.t.dl = dl[i] + r0;
+            t.t.kbeg = d.ks;
+            for (int rt = r0; rt < r1; ++rt) {
+              int kb, ke;
+              steps(d, rt, kb, ke);
+              t.t.kbeg = std::min(t.t.kbeg, kb);
+              t.t.kend = std::max(t.t.kend, ke);
+              t.cost += unit(d, rt, 0, 0);
+            }
+            t.chunks = (t.t.kend + kCh - 1) / kCh - t.t.kbeg / kCh;
+            (t.chunks > 1 ? multi : single).push_back(t);
+          }
+          ++i;
+          continue;
+        }
+        T t{};
+        t.t.u0 = (int32_t)P.units.size();
+        t.chunks = 1;
+        int ks = 0, ne = 0;
+        while (i < lv.size() && ne < kMmPack && ks + lv[i].ks <= kCh && t.t.nu + lv[i].rt <= R) {
+          // a pack's K steps: its supernodes' one after another in its own list
+          for (int rt = 0; rt < lv[i].rt; ++rt) t.cost += unit(lv[i], rt, ne, ks);
+          for (int k = 0; k < lv[i].ks; ++k) t.t.emap |= (uint32_t)ne << (4 * (ks + k));
+          t.t.nu += lv[i].rt;
+          if (ne == 0) t.t.kl = kl[i];
+          ks += lv[i].ks;
+          ++ne;
+          ++i;
+        }
+        t.t.kend = ks;
+        if (ne > 1) {
+          const size_t k0 = P.klist.size();
+          t.t.kl = (int32_t)(k0 / 16);
+          for (size_t q = i - ne; q < i; ++q)
+            for (int k = 0; k < lv[q].ks * 16; ++k) P.klist.push_back(P.klist[(size_t)kl[q] * 16 + k]);
+        }
+        single.push_back(t);
+      }
+      auto longest = [](const T& x, const T& y) { return x.cost > y.cost; };
+      std::stable_sort(multi.begin(), multi.end(), longest);
+      std::stable_sort(single.begin(), single.end(), longest);
+      MmHostPlan::Range r{P.tasks[ver].size(), (int)multi.size(), (int)single.size(), 1};
+      for (const T& t : multi) {
+        r.steps = std::max(r.steps, t.t.kend - t.t.kbeg);
+        P.tasks[ver].push_back(t.t);
+      }
+      for (const T& t : single) P.tasks[ver].push_back(t.t);
+      P.lev[ver].push_back(r);
     }
   }
-  lo[nlev] = list.size();
-  fo[nlev] = tf.size();
-  bo2[nlev] = tb.size();
-  int32_t* ld = nullptr;
-  int2 *tfd = nullptr, *tbd = nullptr;
-  TsSup* sd = nullptr;
-  if (!c->upload(sd, sups.data(), sups.size()) || !c->upload(ld, list.data(), list.size()) ||
-      !c->upload(tfd, tf.data(), tf.size()) || !c->upload(tbd, tb.data(), tb.size()))
-    return false;
-  for (int fi = 0; fi < 2; ++fi) {
-    if (!c->alloc(c->tsA[fi][0], (size_t)aF / 2) || !c->alloc(c->tsA[fi][1], (size_t)aB / 2) ||
-        !c->alloc(c->tsR[fi][0], (size_t)rF) || !c->alloc(c->tsR[fi][1], (size_t)rB))
-      return false;
-  }
-  c->ts_sups = sd;
-  c->ts_n = (int)sups.size();
-  c->ts_levels.assign(nlev, TsLevel{});
-  for (int l = 0; l < nlev; ++l) {
-    TsLevel& L = c->ts_levels[l];
-    L.nsup = (int32_t)(lo[l + 1] - lo[l]);
-    L.list = ld + lo[l];
-    L.ntile_f = (int32_t)(fo[l + 1] - fo[l]);
-    L.tiles_f = tfd + fo[l];
-    L.ntile_b = (int32_t)(bo2[l + 1] - bo2[l]);
-    L.tiles_b = tbd + bo2[l];
-  }
-  for (int fi = 0; fi < 2; ++fi) {
-    const DevFactor& F = fi == 0 ? c->fM : c->fG;
-    ts_split_panels(F, sd, c->ts_n, mtf, true, c->tsA[fi][0], c->tsR[fi][0], c->st);
-    ts_split_panels(F, sd, c->ts_n, mtb, false, c->tsA[fi][1], c->tsR[fi][1], c->st);
-  }
-  c->ts_mtf = mtf;
-  c->ts_mtb = mtb;
-  ts_set_limits();
-  return cudaStreamSynchronize(c->st) == cudaSuccess;
 }
 
-int solve_ts(matex_ctx* c, const DevFactor& F, int fi, int ncols);
+// Both directions' panel tiles of factor fi from its coarse panels (host).
+bool load_mm(matex_ctx* c, int fi, const std::vector<double>& pan) {
+  double* p = nullptr;
+  if (cudaMalloc(&p, sizeof(double) * std::max<size_t>(1, pan.size())) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  bool ok = cudaMemcpy(p, pan.data(), sizeof(double) * pan.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+  for (int dir = 0; ok && dir < 2; ++dir)
+    mm_split_panels(p, (fi == 0 ? c->fM : c->fG).dinv, c->mm, dir == 0, c->mm.A[fi][dir], c->st);
+  ok = cudaStreamSynchronize(c->st) == cudaSuccess && ok;
+  cudaFree(p);
+  return ok;
+}
 
-// Per column count: whether the level solves put the wide supernodes on the
-// tensor cores.  opts.tc_solve 2: always; 0: where the solve pair (level
-// launches, best of three) is at least 5 % faster that way, at each column
-// count the launch-mode tuner measures (1, 2, 4, ..., the buffer width).
-void autotune_ts(matex_ctx* c) {
-  c->ts_by_ncols.assign(c->ldy + 1, 0);
-  c->ts_min_cols = 0;
-  if (c->ts_n == 0) return;
+// The plan and both factors' tiles.  False when there is no room (at most a
+// quarter of the free memory): the solves then stay on the FP64 kernels.
+bool plan_mm(matex_ctx* c, const std::vector<double>& panM, const std::vector<double>& panG) {
+  const Symbolic& S = c->SC;
+  MmHostPlan H[2];
+  for (int dir = 0; dir < 2; ++dir) {
+    build_mm_plan(S, dir == 0, H[dir]);
+    if (H[dir].tiles > INT32_MAX) return false;
+  }
+  const double need = 2.0 * (double)mm_tile_bytes() * (double)(H[0].tiles + H[1].tiles);
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  if (need > 0.25 * (double)free_b || !mm_set_limits()) return false;
+  c->mm.nlev = (int)S.level_ptr.size() - 1;
+  c->mm.nsup = S.nsup;
+  for (int dir = 0; dir < 2; ++dir) {
+    MmSup* sd = nullptr;
+    int4* ud = nullptr;
+    int32_t* kd = nullptr;
+    if (!c->upload(sd, H[dir].sups.data(), H[dir].sups.size()) ||
+        !c->upload(ud, H[dir].units.data(), H[dir].units.size()) ||
+        !c->upload(kd, H[dir].klist.data(), H[dir].klist.size()))
+      return false;
+    c->mm.sups[dir] = sd;
+    c->mm.units[dir] = ud;
+    c->mm.klist[dir] = kd;
+    for (int ver = 0; ver < 2; ++ver) {
+      MmTask* td = nullptr;
+      if (!c->upload(td, H[dir].tasks[ver].data(), H[dir].tasks[ver].size())) return false;
+      c->mm.lev[dir][ver].clear();
+      for (const MmHostPlan::Range& r : H[dir].lev[ver])
+        c->mm.lev[dir][ver].push_back(MmLevel{td + r.t0, r.nmulti, r.nsingle, r.steps});
+    }
+    for (int fi = 0; fi < 2; ++fi)
+      if (!c->alloc(c->mm.A[fi][dir], (size_t)H[dir].tiles * mm_tile_bytes())) return false;
+  }
+  return load_mm(c, 0, panM) && load_mm(c, 1, panG);
+}
+
+// Which solves take the tensor-core kernels.  opts.tc_solve 2: all (one column
+// only when opts.single_column does not force its own kernels); 0: from two
+// columns on, where they measured faster on every grid tried (1,024 to 180k
+// nodes: 1.2 to 1.6 times at two columns, 3.3 times at 16 and 64), and for one
+// column where the pair is at least 5 % faster than the path chosen so far
+// (small grids: 0.049 against 0.062 ms on 1,024 nodes; 0.42 against 0.31 ms on
+// 180k), cached in MATEX_AUTOTUNE_CACHE like the other choices.
+void choose_mm(matex_ctx* c) {
+  c->mm_by_ncols.assign(c->ldy + 1, c->mm_ok ? 1 : 0);
+  if (!c->mm_ok) return;
+  c->mm_by_ncols[0] = 0;
   if (c->opts.tc_solve == 2) {
-    std::fill(c->ts_by_ncols.begin(), c->ts_by_ncols.end(), (int8_t)1);
-    c->ts_min_cols = 1;
+    if (c->opts.single_column == 2) c->mm_by_ncols[1] = 0;
     return;
   }
-  std::vector<int> reps;
-  for (int r = 1; r <= c->ldy; r *= 2) reps.push_back(r);
-  if (reps.back() != c->ldy) reps.push_back(c->ldy);
+  c->mm_by_ncols[1] = 0;
+  if (c->opts.single_column != 0 || c->opts.solve_mode != 2) return;
+  const char* cache = std::getenv("MATEX_AUTOTUNE_CACHE");
+  const std::string key = "mm1:" + tune_key(c);
+  if (cache) {
+    if (FILE* f = std::fopen(cache, "r")) {
+      char line[1024];
+      int found = -1;
+      while (std::fgets(line, sizeof(line), f)) {
+        const std::string l(line);
+        if (l.compare(0, key.size() + 1, key + " ") == 0 && l.size() > key.size() + 1)
+          found = l[key.size() + 1] == '1' ? 1 : 0;
+      }
+      std::fclose(f);
+      if (found >= 0) {
+        c->mm_by_ncols[1] = (int8_t)found;
+        return;
+      }
+    }
+  }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaMemsetAsync(c->Y, 0, sizeof(double) * (size_t)c->n * c->ldy, c->st);
-  cudaMemsetAsync(c->Y2, 0, sizeof(double) * (size_t)c->n * c->ldy, c->st);
-  auto best_of = [&](int K, bool ts) {
-    float best = 1e30f;
+  float best[2] = {1e30f, 1e30f};
+  for (int mm = 0; mm < 2; ++mm) {
+    c->mm_by_ncols[1] = (int8_t)mm;
     for (int rep = 0; rep < 4; ++rep) {
       cudaEventRecord(e0, c->st);
-      if (ts) solve_ts(c, c->fM, 0, K);
-      else solve_inplace(c->fM, c->levels.data(), (int)c->levels.size(), c->Y, c->Y2, c->ldy, K,
-                         c->st, &c->split);
+      solve_cols(c, c->fM, 1);
       cudaEventRecord(e1, c->st);
       cudaEventSynchronize(e1);
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
-      if (rep > 0) best = std::min(best, ms);  // the first is the warm-up
+      if (rep > 0) best[mm] = std::min(best[mm], ms);  // the first is the warm-up
     }
-    return best;
-  };
-  std::vector<int8_t> use(reps.size(), 0);
-  for (size_t b = 0; b < reps.size(); ++b) use[b] = best_of(reps[b], true) < 0.95f * best_of(reps[b], false);
+  }
+  c->mm_by_ncols[1] = cudaGetLastError() == cudaSuccess && best[1] < 0.95f * best[0];
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  for (size_t b = 0; b < reps.size(); ++b) {
-    const int lo = reps[b];
-    const int hi = b + 1 < reps.size() ? reps[b + 1] - 1 : c->ldy;
-    for (int nc = lo; nc <= hi; ++nc) c->ts_by_ncols[nc] = use[b];
-    if (use[b] && c->ts_min_cols == 0) c->ts_min_cols = lo;
+  if (cache) {
+    if (FILE* f = std::fopen(cache, "a")) {
+      std::fprintf(f, "%s %d\n", key.c_str(), (int)c->mm_by_ncols[1]);
+      std::fclose(f);
+    }
   }
-  cudaGetLastError();
-}
-
-// The level-by-level solve pair with the wide supernodes' products on the
-// tensor cores (factor index fi: 0 = C + gamma G, 1 = G); returns launches.
-int solve_ts(matex_ctx* c, const DevFactor& F, int fi, int ncols) {
-  const int nlev = (int)c->levels_n.size();
-  int launches = 0;
-  int32_t* err = c->d_count + 1;
-  for (int l = 0; l < nlev; ++l) {
-    solve_level(true, F, c->levels_n[l], c->Y, c->Y2, c->ldy, ncols, c->st, &c->split);
-    ts_solve_level(F, c->ts_sups, c->ts_levels[l], true, c->tsA[fi][0], c->tsR[fi][0], c->Y, c->Y2,
-                   c->ldy, ncols, err, c->st);
-    launches += 3;
-  }
-  for (int l = nlev - 1; l >= 0; --l) {
-    solve_level(false, F, c->levels_n[l], c->Y, c->Y2, c->ldy, ncols, c->st, &c->split);
-    ts_solve_level(F, c->ts_sups, c->ts_levels[l], false, c->tsA[fi][1], c->tsR[fi][1], c->Y, c->Y2,
-                   c->ldy, ncols, err, c->st);
-    launches += 3;
-  }
-  return launches;
 }
 
 int solve_cols(matex_ctx* c, const DevFactor& F, int ncols) {
   if (ncols <= 0) return 0;
+  // factors with panel digits (the trapezoidal one has none)
+  const int fi = F.pan_cm == c->fM.pan_cm ? 0 : F.pan_cm == c->fG.pan_cm ? 1 : -1;
+  if (fi >= 0 && !c->mm_by_ncols.empty() && c->mm_by_ncols[std::min(ncols, c->ldy)])
+    return solve_mm(F.abort, c->mm, fi, c->Y, c->Y2, c->ldy, ncols, c->st);
   // one column: the single-column level kernels (any factor of this
   // symbolic structure: C + gamma G, G, the trapezoidal one)
   if (ncols == 1 && c->k1_use && F.sup_first == c->fM.sup_first)
     return solve_k1(F, c->k1, c->Y, c->Y2, c->ldy, c->st);
   int mode = c->opts.solve_mode;
   if (mode == 2) mode = c->mode_by_ncols.empty() ? 0 : c->mode_by_ncols[std::min(ncols, c->ldy)];
-  const int fi = F.pan_cm == c->fM.pan_cm ? 0 : F.pan_cm == c->fG.pan_cm ? 1 : -1;
-  if (mode == 1 && fi >= 0 && c->ts_n > 0 && !c->ts_by_ncols.empty() &&
-      c->ts_by_ncols[std::min(ncols, c->ldy)])
-    return solve_ts(c, F, fi, ncols);
   if (mode == 1)
     return solve_inplace(F, c->levels.data(), (int)c->levels.size(), c->Y, c->Y2, c->ldy, ncols,
                          c->st, &c->split);
@@ -2398,16 +2439,21 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   CsrSym A{n, g_rowptr, g_col, g_val};
   std::vector<int32_t> nd;
   std::string e = nested_dissection(A, nd);
-  if (e.empty()) e = symbolic_analysis(A, nd, o.max_width, c->S);
+  // the tensor-core solves are on unless another path is asked for
+  const bool want_mm = o.tc_solve != 1 && o.solve_mode != 0;
+  if (e.empty()) e = symbolic_analysis(A, nd, o.max_width, c->S, &c->SC);
   if (!e.empty()) { c->err = e; g_setup_err = e; delete c; return MATEX_ERR_ARG; }
   c->setup_stats.setup_order_ms = now_ms() - t;
   t = now_ms();
   Numeric NM, NG;
+  std::vector<double> mm_panM, mm_panG;
   {
     // the two factorisations are independent: run them side by side
     std::string eg;
-    std::thread tg([&] { eg = numeric_ldlt(A, nullptr, 1.0, c->S, NG); });
-    e = numeric_ldlt(A, cap, gamma, c->S, NM);
+    std::thread tg([&] {
+      eg = numeric_ldlt(A, nullptr, 1.0, c->S, NG, &c->SC, want_mm ? &mm_panG : nullptr);
+    });
+    e = numeric_ldlt(A, cap, gamma, c->S, NM, &c->SC, want_mm ? &mm_panM : nullptr);
     tg.join();
     if (e.empty()) e = eg;
   }
@@ -2675,7 +2721,6 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   if (!c->replay.empty()) ok = ok && c->upload(c->replay_d, c->replay.data(), c->replay.size());
   // work buffers
   c->ldy = roundup8(std::max({Kmax, 8, std::min<int>(n_groups, 256)}));
-  c->ts_minw = o.tc_solve == 1 ? 0 : (o.tc_min_width > 0 ? o.tc_min_width : kTsMinWidth);
   ok = ok && plan_levels(c);
   c->nchunks = (int)((n + kChunk - 1) / kChunk);
   const size_t G = (size_t)c->g_slots;
@@ -2801,17 +2846,23 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   }
   if (o.solve_mode == 2 && o.col_block == 0) autotune_levels(c);
   if (o.solve_mode == 2) autotune_solve(c);
-  if (c->ts_minw > 0 && o.solve_mode != 0) {
-    if (plan_ts(c)) autotune_ts(c);
-    cudaGetLastError();
-  }
-  c->setup_stats.tc_solve_supernodes = c->ts_n;
-  c->setup_stats.tc_solve_min_cols = c->ts_min_cols;
   if (o.single_column == 2 || (o.single_column == 0 && o.solve_mode == 2)) {
     autotune_k1(c);
     cudaGetLastError();
   }
   c->setup_stats.single_column = c->k1_use ? 1 : 0;
+  if (want_mm) {
+    c->mm_ok = plan_mm(c, mm_panM, mm_panG);
+    cudaGetLastError();
+    choose_mm(c);
+    cudaGetLastError();
+  }
+  if (c->mm_ok) {
+    const int minw = o.tc_min_width > 0 ? o.tc_min_width : 64;
+    for (int32_t s = 0; s < S.nsup; ++s)
+      c->setup_stats.tc_solve_supernodes += S.sup_first[s + 1] - S.sup_first[s] >= minw;
+    c->setup_stats.tc_solve_min_cols = c->mm_by_ncols[1] ? 1 : 2;
+  }
   if (o.resident != 1 && o.krylov != 2 && o.tape == 0 && o.tail_eps == 0.0 &&
       n <= kResidentMaxN) {
     // resident rounds: one CTA's solve pair against the batched path's
@@ -2900,7 +2951,8 @@ matex_status matex_set_caps(matex_ctx* c, const double* cap) {
   const double t = now_ms();
   CsrSym A{c->n, c->g_rowptr_h.data(), c->g_col_h.data(), c->g_val_h.data()};
   Numeric NM;
-  std::string e = numeric_ldlt(A, cap, c->gamma, c->S, NM);
+  std::vector<double> mm_pan;
+  std::string e = numeric_ldlt(A, cap, c->gamma, c->S, NM, &c->SC, c->mm_ok ? &mm_pan : nullptr);
   if (!e.empty()) return fail(c, MATEX_ERR_NOT_SPD, e);
   if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check(c, "set_caps sync");
   std::vector<double> cp(c->n);
@@ -2914,12 +2966,7 @@ matex_status matex_set_caps(matex_ctx* c, const double* cap) {
             cudaMemcpy(c->c_perm, cp.data(), sizeof(double) * c->n, cudaMemcpyHostToDevice) ==
                 cudaSuccess;
   if (!ok) return cuda_check(c, "set_caps upload");
-  if (c->ts_n > 0) {
-    // the tensor-core slices of the refactored C + gamma G
-    ts_split_panels(c->fM, c->ts_sups, c->ts_n, c->ts_mtf, true, c->tsA[0][0], c->tsR[0][0], c->st);
-    ts_split_panels(c->fM, c->ts_sups, c->ts_n, c->ts_mtb, false, c->tsA[0][1], c->tsR[0][1], c->st);
-    if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check(c, "set_caps slices");
-  }
+  if (c->mm_ok && !load_mm(c, 0, mm_pan)) return cuda_check(c, "set_caps tiles");
   if (c->resident_ok) {
     // the resident copy of the refactored C + gamma G
     resident_store(c->fM, c->rsup, c->S.nsup, const_cast<double*>(c->rM.fpan),
@@ -3345,6 +3392,150 @@ extern "C" matex_status matex_host_single_column_plan(int64_t n, const int64_t* 
   return MATEX_OK;
 }
 
+extern "C" matex_status matex_host_tensor_plan(int64_t n, const int64_t* rowptr, const int32_t* col,
+                                               const double* val, const double* dshift, double alpha,
+                                               int32_t max_width, int32_t version, int32_t cluster,
+                                               int32_t ncols, const double* b, double* x,
+                                               int64_t* info) {
+  g_setup_err.clear();
+  if (n <= 0 || !rowptr || !col || !val || version < 0 || version > 1 || cluster < 1 || cluster > 8 ||
+      ncols < 0 || (ncols > 0 && (!b || !x))) {
+    g_setup_err = "bad arguments";
+    return MATEX_ERR_ARG;
+  }
+  CsrSym A{n, rowptr, col, val};
+  std::vector<int32_t> nd;
+  Symbolic S, C;
+  std::string e = nested_dissection(A, nd);
+  if (e.empty()) e = symbolic_analysis(A, nd, max_width > 0 ? max_width : 1024, S, &C);
+  if (!e.empty()) { g_setup_err = e; return MATEX_ERR_ARG; }
+  Numeric F;
+  std::vector<double> pan;
+  e = numeric_ldlt(A, dshift, alpha, S, F, &C, &pan);
+  if (!e.empty()) { g_setup_err = e; return MATEX_ERR_NOT_SPD; }
+  constexpr int kCh = 8;
+  const int nlev = (int)C.level_ptr.size() - 1;
+  MmHostPlan H[2];
+  build_mm_plan(C, true, H[0]);
+  build_mm_plan(C, false, H[1]);
+  int64_t errors = 0, ntasks = 0, nmulti = 0;
+  // Y and Y2, ncols columns a node
+  std::vector<double> Y((size_t)n * ncols), Y2((size_t)n * ncols, 0.0), part, piece;
+  for (int64_t k = 0; k < n; ++k)
+    for (int32_t q = 0; q < ncols; ++q) Y[k * ncols + q] = b[(int64_t)q * n + S.perm[k]];
+  for (int dir = 0; dir < 2; ++dir) {
+    const bool fwd = dir == 0;
+    const MmHostPlan& P = H[dir];
+    std::vector<char> seen((size_t)P.tiles, 0);
+    // panel entry (row r, term k) of supernode d's product, as the tiles hold it
+    auto entry = [&](const MmSup& d, int64_t r, int64_t k) {
+      if (r >= (fwd ? d.ld : d.w) || k >= (fwd ? d.w : d.ld)) return 0.0;
+      const double v = fwd ? pan[d.pan + k * d.ld + r] : pan[d.pan + r * d.ld + k];
+      if (fwd) return r < d.w ? v * F.dinv[d.f + r] : -v;
+      return k < d.w ? v : -v;
+    };
+    for (int step = 0; step < nlev; ++step) {
+      const MmHostPlan::Range& R = P.lev[version][fwd ? step : nlev - 1 - step];
+      for (int ti = 0; ti < R.nmulti + R.nsingle; ++ti) {
+        const MmTask& tk = P.tasks[version][R.t0 + ti];
+        const bool multi = ti < R.nmulti;
+        ++ntasks;
+        nmulti += multi;
+        if (tk.nu > (multi ? kMmRowsNarrow : kMmRowsWide) || tk.nu <= 0) ++errors;
+        if (multi && tk.kend - tk.kbeg > R.steps) ++errors;
+        part.assign((size_t)tk.nu * 8 * ncols, 0.0);
+        const int cs = multi ? cluster : 1;
+        for (int rank = 0; rank < cs; ++rank) {
+          const int ka = tk.kbeg + (tk.kend - tk.kbeg) * rank / cs;
+          const int kz = tk.kbeg + (tk.kend - tk.kbeg) * (rank + 1) / cs;
+          const int chb = ka / kCh, che = ka < kz ? (kz - 1) / kCh + 1 : chb;
+          if (!multi && che - chb != 1) ++errors;
+          for (int ch = chb; ch < che; ++ch) {
+            const int k0 = std::max(ka, ch * kCh), k1 = std::min(kz, (ch + 1) * kCh);
+            piece.assign((size_t)kCh * 16 * ncols, 0.0);
+            for (int ks = k0; ks < k1; ++ks)
+              for (int t = 0; t < 16; ++t) {
+                const int32_t r = P.klist[(int64_t)(tk.kl + ks) * 16 + t];
+                if (r < 0) continue;
+                const double* src = (!fwd && !(r & kMmAdd) ? Y2 : Y).data() + (int64_t)(r & (kMmAdd - 1)) * ncols;
+                std::copy(src, src + ncols, &piece[((ks - k0) * 16 + t) * (size_t)ncols]);
+              }
+            for (int u = 0; u < tk.nu; ++u) {
+              const int4& un = P.units[tk.u0 + u];
+              const int slot = un.z >> 16;
+              const int kb = std::max(un.y & 0xffff, k0 - slot), ke = std::min(un.y >> 16, k1 - slot);
+              // the supernode of the unit's tiles
+              size_t lo = 0, hi = P.sups.size() - 1;
+              while (lo < hi) {
+                const size_t mid = (lo + hi + 1) / 2;
+                if (P.sups[mid].a <= un.x) lo = mid;
+                else hi = mid - 1;
+              }
+              const MmSup& d = P.sups[lo];
+              const int64_t rt = (un.x - d.a) / d.ks;
+              for (int r = 0; r < 8; ++r)
+                if (P.klist[(int64_t)d.dl * 8 + rt * 8 + r] !=
+                    (multi ? P.klist[((int64_t)tk.dl + u) * 8 + r] : P.klist[(int64_t)d.dl * 8 + rt * 8 + r]))
+                  ++errors;
+              for (int ks = kb; ks < ke; ++ks) {
+                if (((tk.emap >> (4 * ((slot + ks) & 7))) & 15) != (uint32_t)(un.z & 0xffff)) ++errors;
+                if (slot + ks - k0 < 0 || slot + ks - k0 >= kCh) { ++errors; continue; }
+                if (seen[un.x + ks]++) ++errors;
+                for (int r = 0; r < 8; ++r)
+                  for (int t = 0; t < 16; ++t) {
+                    const double v = entry(d, rt * 8 + r, (int64_t)ks * 16 + t);
+                    const double* bp = &piece[((slot + ks - k0) * 16 + t) * (size_t)ncols];
+                    for (int32_t q = 0; q < ncols; ++q) part[(u * 8 + r) * (size_t)ncols + q] += v * bp[q];
+                  }
+              }
+            }
+          }
+        }
+        for (int u = 0; u < tk.nu; ++u) {
+          const int4& un = P.units[tk.u0 + u];
+          size_t lo = 0, hi = P.sups.size() - 1;
+          while (lo < hi) {
+            const size_t mid = (lo + hi + 1) / 2;
+            if (P.sups[mid].a <= un.x) lo = mid;
+            else hi = mid - 1;
+          }
+          const MmSup& d = P.sups[lo];
+          const int64_t rt = (un.x - d.a) / d.ks;
+          for (int r = 0; r < 8; ++r) {
+            const int32_t dst = P.klist[(int64_t)d.dl * 8 + rt * 8 + r];
+            if (dst < 0) continue;
+            double* out = (fwd && !(dst & kMmAdd) ? Y2 : Y).data() + (int64_t)(dst & (kMmAdd - 1)) * ncols;
+            for (int32_t q = 0; q < ncols; ++q) {
+              const double v = part[(u * 8 + r) * (size_t)ncols + q];
+              if (fwd && (dst & kMmAdd)) out[q] += v;
+              else out[q] = v;
+            }
+          }
+        }
+      }
+    }
+    // a tile no unit takes must hold zeros only (the triangle of L_ss^{-1})
+    for (const MmSup& d : P.sups)
+      for (int64_t t = 0; t < (int64_t)d.rt * d.ks; ++t)
+        if (!seen[d.a + t])
+          for (int64_t r = t / d.ks * 8; r < t / d.ks * 8 + 8; ++r)
+            for (int64_t k = t % d.ks * 16; k < t % d.ks * 16 + 16; ++k) errors += entry(d, r, k) != 0.0;
+  }
+  for (int64_t k = 0; k < n; ++k)
+    for (int32_t q = 0; q < ncols; ++q) x[(int64_t)q * n + S.perm[k]] = Y[k * ncols + q];
+  if (info) {
+    info[0] = C.nsup;
+    info[1] = ntasks;
+    info[2] = nmulti;
+    info[3] = errors;
+  }
+  if (errors) {
+    g_setup_err = "tensor-core plan: " + std::to_string(errors) + " mapping errors";
+    return MATEX_ERR_STATE;
+  }
+  return MATEX_OK;
+}
+
 // ---------------------------------------------------------------------------
 // Allocation-free solve.  Code that must not touch the CUDA allocator (it runs
 // where cudaMalloc is forbidden or would deadlock, e.g. inside another
@@ -3494,7 +3685,7 @@ matex_status tr_prepare(matex_ctx* c, double h) {
   const double t0 = now_ms();
   CsrSym A{n, c->g_rowptr_h.data(), c->g_col_h.data(), c->g_val_h.data()};
   Numeric NT;
-  const std::string e = numeric_ldlt(A, c->c_host.data(), 0.5 * h, c->S, NT);
+  const std::string e = numeric_ldlt(A, c->c_host.data(), 0.5 * h, c->S, NT, &c->SC);
   if (!e.empty()) return fail(c, MATEX_ERR_NOT_SPD, e);
   if (!c->fT.dinv) {
     double *d, *pc, *pr;

@@ -1,9 +1,8 @@
 // Building blocks of the error-free bf16 tensor-core products (the Ozaki
 // scheme: Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
 // multiplication by using fast routines of matrix multiplication and its
-// applications", Numer. Algorithms 59, 2012) shared by the recombination and
-// the wide panels of the triangular solves: the base-64 digit split of FP64
-// values, the K-major core-matrix tile layout, and tcgen05 / bulk-copy /
+// applications", Numer. Algorithms 59, 2012) used by the recombination: the
+// base-64 digit split of FP64 values, the K-major core-matrix tile layout, and tcgen05 / bulk-copy /
 // mbarrier operations as inline PTX.
 //
 // A K step is 32 values of the reduction (two MMAs of K = 16); an operand

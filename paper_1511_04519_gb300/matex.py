@@ -77,7 +77,8 @@ EXPORTS = ["matex_default_opts", "matex_setup", "matex_run", "matex_run_host", "
            "matex_debug_inject_wait", "matex_solve_noalloc", "matex_grad", "matex_set_caps",
            "matex_get_autotune", "matex_batch_create", "matex_batch_run", "matex_batch_last_error",
            "matex_batch_destroy", "matex_measure_fp64_peak", "matex_tr_run",
-           "matex_time_solve", "matex_get_level_blocks", "matex_solve_resident"]
+           "matex_time_solve", "matex_get_level_blocks", "matex_solve_resident",
+           "matex_host_tensor_plan"]
 
 
 def _load():
