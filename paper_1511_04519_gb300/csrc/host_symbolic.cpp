@@ -178,11 +178,13 @@ void keep_supernodes(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
   offrows.swap(rows2);
 }
 
-// Supernodes renumbered, every parent's children with the largest subtree
-// first: the small ones end up adjacent to their parent.  Only the numbering
-// changes, no panel.
+// Supernodes renumbered: every parent's children with the largest subtree
+// first, so that the small ones end up adjacent to their parent, and those of
+// level l0 and above (lev) after all others.  Only the numbering changes, no
+// panel.
 void order_children(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
-                    std::vector<int32_t>& col2sup, std::vector<int64_t>& zeros) {
+                    std::vector<int32_t>& col2sup, std::vector<int64_t>& zeros,
+                    std::vector<int32_t>& lev, int32_t l0) {
   const int32_t ns = S.nsup;
   std::vector<int64_t> size(ns);
   std::vector<std::vector<int32_t>> kids(ns);
@@ -205,7 +207,8 @@ void order_children(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
     stack.insert(stack.end(), kids[s].begin(), kids[s].end());
   }
   std::reverse(order.begin(), order.end());
-  std::vector<int32_t> first(ns + 1, 0), map(S.n), pos(ns), perm(S.n), par(ns);
+  std::stable_partition(order.begin(), order.end(), [&](int32_t s) { return lev[s] < l0; });
+  std::vector<int32_t> first(ns + 1, 0), map(S.n), pos(ns), perm(S.n), par(ns), lv(ns);
   std::vector<std::vector<int32_t>> rows(ns);
   std::vector<int64_t> z(ns);
   for (int32_t k = 0; k < ns; ++k) {
@@ -213,6 +216,7 @@ void order_children(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
     pos[s] = k;
     first[k + 1] = first[k] + w;
     z[k] = zeros[s];
+    lv[k] = lev[s];
     for (int32_t j = 0; j < w; ++j) {
       map[S.sup_first[s] + j] = first[k] + j;
       perm[first[k] + j] = S.perm[S.sup_first[s] + j];
@@ -232,6 +236,60 @@ void order_children(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
   for (int64_t k = 0; k < S.n; ++k) S.iperm[S.perm[k]] = (int32_t)k;
   offrows.swap(rows);
   zeros.swap(z);
+  lev.swap(lv);
+}
+
+// Widest merged top: every level taken away saves two dependent launches
+// (level solves: 4.5 to 8 us each).  Pair of 8 columns, 512 against none: 77
+// against 99 us on 10,000 nodes, 141 against 164 us on 39,711 (1,024: 70 and
+// 134); the solution's error on the latter 2.6e-15 against 2.2e-15 with none,
+// 3.0e-15 with 1,024 (entries of larger inverses), which set the limit.
+constexpr int64_t kTopWidth = 512;
+constexpr int64_t kTopMinN = 8192;  // smaller grids keep their panels for the resident rounds
+
+// Level of every supernode: 0 for leaves, else one above its highest child.
+std::vector<int32_t> sup_levels(const Symbolic& S) {
+  std::vector<int32_t> lev(S.nsup, 0);
+  for (int32_t s = 0; s < S.nsup; ++s)
+    if (S.sup_parent[s] >= 0) lev[S.sup_parent[s]] = std::max(lev[S.sup_parent[s]], lev[s] + 1);
+  return lev;
+}
+
+// The lowest level from which the tree above is at most `cap` columns and has
+// one root: those supernodes may become one (number of levels: none).
+int32_t top_level(const Symbolic& S, const std::vector<int32_t>& lev, int64_t cap) {
+  int32_t nlev = 0, roots = 0;
+  for (int32_t s = 0; s < S.nsup; ++s) {
+    nlev = std::max(nlev, lev[s] + 1);
+    roots += S.sup_parent[s] < 0;
+  }
+  if (roots != 1) return nlev;
+  std::vector<int64_t> w(nlev, 0);
+  for (int32_t s = 0; s < S.nsup; ++s) w[lev[s]] += S.sup_first[s + 1] - S.sup_first[s];
+  int32_t l = nlev;
+  for (int64_t sum = 0; l > 0 && sum + w[l - 1] <= cap; --l) sum += w[l - 1];
+  return l;
+}
+
+// The supernodes of level l0 and above, numbered last, as one.
+void merge_top(Symbolic& S, std::vector<std::vector<int32_t>>& offrows, std::vector<int32_t>& col2sup,
+               std::vector<int64_t>& zeros, const std::vector<int32_t>& lev, int32_t l0) {
+  std::vector<char> gone(S.nsup, 0);
+  std::vector<int32_t> first(S.sup_first.begin(), S.sup_first.end() - 1);
+  int32_t root = -1;
+  int64_t w = 0, have = 0;
+  for (int32_t s = 0; s < S.nsup; ++s) {
+    if (lev[s] < l0) continue;
+    const int64_t ws = S.sup_first[s + 1] - S.sup_first[s];
+    if (root < 0) first[S.nsup - 1] = S.sup_first[s];
+    root = s;
+    w += ws;
+    have += ws * (ws + 1) / 2 + ws * (int64_t)offrows[s].size() - zeros[s];
+    gone[s] = s != S.nsup - 1;
+  }
+  if (root < 0) return;
+  zeros[root] = w * (w + 1) / 2 - have;
+  keep_supernodes(S, offrows, col2sup, zeros, first, gone);
 }
 
 // Amalgamation for the tensor-core solves (k_sptrsv_mma.cu), whose unit of
@@ -518,11 +576,21 @@ std::string symbolic_analysis(const CsrSym& A, const std::vector<int32_t>& nd_pe
     }
     keep_supernodes(S, offrows, col2sup, zeros, first, gone);
   }
-  order_children(S, offrows, col2sup, zeros);
+  // The top levels hold few supernodes whose separators are nearly dense in
+  // each other: as one supernode of at most kTopWidth columns they cost one
+  // launch per direction instead of one each.
+  std::vector<int32_t> lev = sup_levels(S);
+  const int32_t l0 = top_level(S, lev, std::min<int64_t>({max_width, kTopWidth, n / 8}));
+  order_children(S, offrows, col2sup, zeros, lev, l0);
+  if (n > kTopMinN) {
+    merge_top(S, offrows, col2sup, zeros, lev, l0);
+    lev.clear();
+  }
   if (coarse) {
     *coarse = S;
     std::vector<std::vector<int32_t>> rows = offrows;
     std::vector<int32_t> c2s = col2sup;
+    if (!lev.empty()) merge_top(*coarse, rows, c2s, zeros, lev, l0);
     amalgamate_tiled(*coarse, rows, c2s, zeros, max_width);
     lay_out(*coarse, rows);
   }
