@@ -276,7 +276,7 @@ adj_small_kernel(AdjRound ar, double gamma, const double* __restrict__ ybo, int 
     sh.E[i * kMaxM + j] = i == j ? 1.0 : 0.0;
   }
   __syncthreads();
-  SD1::lu_solve(w1.V, sh.E, m, &w1.piv);
+  SD1::lu_solve(w1.V, sh.E, m, &w1.piv, w1.inv);
   // T1 = Hbar Htilde^{-T}
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
     const int i = e / m, j = e - i * m;

@@ -155,36 +155,86 @@ __global__ void basis_scale_kernel(double* __restrict__ Vb, int64_t vstride,
   Vb[g * vstride + (int64_t)wslot * n + x] *= scale[q];
 }
 
-__global__ void start_finish_kernel(const double* __restrict__ partials, int nchunks, int K,
-                                    SmallState ss, const int32_t* __restrict__ groups,
-                                    int32_t* iter_out, int32_t* iter_grp, int32_t* iter_count) {
-  // one thread per column, then a serial compaction by thread 0 (K <= a few hundred)
-  const int q = threadIdx.x;
-  for (int c = q; c < K; c += blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < nchunks; ++k) s += partials[(int64_t)c * nchunks + k];
+// The columns p < K_in (list iter_in, or all in order) with status 0, kept in
+// order in iter_out with their slots in iter_grp, their number in *count, by
+// one CTA.  With expected >= 0 (a recorded run, whose launches were sized for
+// that many) another number raises ca.flag and points the surplus entries at
+// column 0, so that the rest of the replay, whose result is discarded, stays in
+// range.
+__device__ void compact_columns(SmallState ss, const CompactArgs& ca, const int32_t* iter_in, int K_in) {
+  __shared__ int warp_cnt[33];
+  __shared__ int base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  if (threadIdx.x == 0) base = 0;
+  for (int p0 = 0; p0 < K_in; p0 += blockDim.x) {
+    const int p = p0 + (int)threadIdx.x;
+    const int q = p < K_in ? (iter_in ? iter_in[p] : p) : 0;
+    const bool live = p < K_in && __ldcg(ss.status + q) == 0;
+    const unsigned mask = __ballot_sync(0xffffffffu, live);
+    if (lane == 0) warp_cnt[warp] = __popc(mask);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int s = base;
+      for (int w = 0; w < nw; ++w) {
+        const int c = warp_cnt[w];
+        warp_cnt[w] = s;
+        s += c;
+      }
+      base = s;
+    }
+    __syncthreads();
+    if (live) {
+      const int k = warp_cnt[warp] + __popc(mask & ((1u << lane) - 1u));
+      ca.iter_grp[k] = ca.slots[q];
+      ca.iter_out[k] = q;
+    }
+    __syncthreads();
+  }
+  const int cnt = base;
+  if (threadIdx.x == 0) {
+    *ca.count = cnt;
+    if (ca.expected >= 0 && cnt != ca.expected) *ca.flag = 1;
+  }
+  if (ca.expected > cnt)
+    for (int k = cnt + (int)threadIdx.x; k < ca.expected; k += blockDim.x) {
+      ca.iter_out[k] = 0;
+      ca.iter_grp[k] = ca.slots[0];
+    }
+}
+
+// True in the CTA of the grid that arrives last, whose threads then see what
+// the others wrote; the counter is zero again afterwards.
+__device__ bool last_cta(int32_t* arrived) {
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(arrived, 1) == (int)gridDim.x - 1;
+    if (last) *arrived = 0;
+    __threadfence();
+  }
+  __syncthreads();
+  return last != 0;
+}
+
+__global__ void __launch_bounds__(kRedThreads)
+start_finish_kernel(const double* __restrict__ partials, int nchunks, int K, SmallState ss,
+                    CompactArgs ca) {
+  __shared__ double red[32];
+  const int c = blockIdx.x;
+  double acc = 0.0;
+  for (int k = threadIdx.x; k < nchunks; k += blockDim.x) acc += partials[(int64_t)c * nchunks + k];
+  const double s = block_sum(acc, red);
+  for (int i = threadIdx.x; i < kMaxB * kMaxM; i += blockDim.x) ss.Ht[(int64_t)c * kMaxB * kMaxM + i] = 0.0;
+  if (threadIdx.x == 0) {
     const double beta = sqrt(s);
     ss.beta[c] = beta;
     ss.m[c] = 0;
-    for (int i = 0; i < kMaxB * kMaxM; ++i) ss.Ht[(int64_t)c * kMaxB * kMaxM + i] = 0.0;
-    if (beta <= 1e-300) {
-      ss.status[c] = 4;
-      ss.scale[c] = 0.0;
-    } else {
-      ss.status[c] = 0;
-      ss.scale[c] = 1.0 / beta;
-    }
+    const bool quiet = beta <= 1e-300;
+    ss.status[c] = quiet ? 4 : 0;
+    ss.scale[c] = quiet ? 0.0 : 1.0 / beta;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int cnt = 0;
-    for (int c = 0; c < K; ++c)
-      if (ss.status[c] == 0) {
-        iter_grp[cnt] = groups[c];
-        iter_out[cnt++] = c;
-      }
-    *iter_count = cnt;
-  }
+  if (last_cta(ca.arrived)) compact_columns(ss, ca, nullptr, K);
 }
 
 __global__ void reduce_dots_kernel(const double* __restrict__ partials, int nchunks, int nb,
@@ -206,28 +256,13 @@ __global__ void reduce_dots_kernel(const double* __restrict__ partials, int nchu
   }
 }
 
-__global__ void __launch_bounds__(kSmallThreads)
+__global__ void __launch_bounds__(kTeamThreads)
 residual_kernel(SmallState ss, RoundCols rc, const int32_t* __restrict__ iter, int j, double gamma,
-                double tol, int m_max, const int32_t* __restrict__ replay) {
+                double tol, int m_max, const int32_t* __restrict__ replay, CompactArgs ca) {
   extern __shared__ double smem_raw[];
-  SmallShared& sh = *reinterpret_cast<SmallShared*>(smem_raw);
-  residual_column(ss, rc, iter[blockIdx.x], j, gamma, tol, m_max, replay, sh);
-}
-
-__global__ void compact_kernel(SmallState ss, const int32_t* __restrict__ groups,
-                               const int32_t* __restrict__ iter_in, int K_in,
-                               int32_t* __restrict__ iter_out, int32_t* __restrict__ iter_grp,
-                               int32_t* __restrict__ count) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int c = 0;
-  for (int p = 0; p < K_in; ++p) {
-    const int q = iter_in[p];
-    if (ss.status[q] == 0) {
-      iter_grp[c] = groups[q];
-      iter_out[c++] = q;
-    }
-  }
-  *count = c;
+  SmallShared<CtaTeam::kWorkers>& sh = *reinterpret_cast<SmallShared<CtaTeam::kWorkers>*>(smem_raw);
+  residual_column<CtaTeam>(ss, rc, iter[blockIdx.x], j, gamma, tol, m_max, replay, 0.0, sh);
+  if (last_cta(ca.arrived)) compact_columns(ss, ca, iter, gridDim.x);
 }
 
 __global__ void record_kernel(SmallState ss, RoundCols rc, int K, int32_t* m_rec, int32_t* st_rec) {
@@ -237,33 +272,28 @@ __global__ void record_kernel(SmallState ss, RoundCols rc, int K, int32_t* m_rec
   st_rec[rc.segid[q]] = ss.status[q];
 }
 
-__global__ void __launch_bounds__(kSmallThreads)
+__global__ void __launch_bounds__(kTeamThreads)
 coef_kernel(SmallState ss, RoundCols rc, double gamma, double dt_out, double* __restrict__ coef,
             int ldo, double* __restrict__ yend, double tail_eps, const double* __restrict__ pbound,
             int32_t* __restrict__ tcut) {
   extern __shared__ double smem_raw[];
-  SmallShared& sh = *reinterpret_cast<SmallShared*>(smem_raw);
+  SmallShared<CtaTeam::kWorkers>& sh = *reinterpret_cast<SmallShared<CtaTeam::kWorkers>*>(smem_raw);
   if (threadIdx.x == 0) sh.cm = 0;  // no residual test ran in this CTA
   __syncthreads();
-  coef_column(ss, rc, blockIdx.x, gamma, dt_out, coef, ldo, yend, tail_eps, pbound, tcut, sh);
+  coef_column<CtaTeam>(ss, rc, blockIdx.x, gamma, dt_out, coef, ldo, yend, tail_eps, pbound, tcut, sh);
 }
 
+// One matrix per CTA: 64 threads up to 8 x 8 (an entry each), 128 beyond.
 __global__ void __launch_bounds__(kSmallThreads)
 expm_batch_kernel(int m, const double* __restrict__ A, const double* __restrict__ h,
                   double* __restrict__ E) {
-  extern __shared__ double smem_raw[];
-  SmallShared& sh = *reinterpret_cast<SmallShared*>(smem_raw);
+  __shared__ ExpmWork w;
+  __shared__ double H[kMat];
   const int b = blockIdx.x;
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int i = e / m, j = e - i * m;
-    sh.H[i * kLd + j] = A[(int64_t)b * m * m + e];
-  }
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) H[(e / m) * kLd + e % m] = A[(int64_t)b * m * m + e];
   __syncthreads();
-  expm_dev(sh.H, h[b], sh.E, m, sh.w);
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int i = e / m, j = e - i * m;
-    E[(int64_t)b * m * m + e] = sh.E[i * kLd + j];
-  }
+  expm_dev(H, h[b], H, m, w);
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) E[(int64_t)b * m * m + e] = H[(e / m) * kLd + e % m];
 }
 
 }  // namespace
@@ -315,10 +345,9 @@ void basis_scale(double* Vbase, int64_t vstride, const int32_t* groups, const in
   basis_scale_kernel<<<grid, 256, 0, st>>>(Vbase, vstride, groups, iter, wslot, scale, n);
 }
 
-void start_finish(const double* partials, int nchunks, int K, SmallState ss, const int32_t* groups,
-                  int32_t* iter_out, int32_t* iter_grp, int32_t* iter_count, cudaStream_t st) {
-  start_finish_kernel<<<1, 256, 0, st>>>(partials, nchunks, K, ss, groups, iter_out, iter_grp,
-                                         iter_count);
+void start_finish(const double* partials, int nchunks, int K, SmallState ss, const CompactArgs& ca,
+                  cudaStream_t st) {
+  start_finish_kernel<<<K, kRedThreads, 0, st>>>(partials, nchunks, K, ss, ca);
 }
 
 void reduce_dots(const double* partials, int nchunks, int K, int nb, const int32_t* iter,
@@ -340,18 +369,6 @@ __global__ void apply_A_kernel(double* __restrict__ Vb, int64_t vstride,
   Vb[(int64_t)iter_grp[blockIdx.y] * vstride + (int64_t)jdst * n + i] = -gv / c[i];
 }
 
-__global__ void expect_count_kernel(const int32_t* __restrict__ count, int expected,
-                                    int32_t* __restrict__ iter, int32_t* __restrict__ iter_grp,
-                                    const int32_t* __restrict__ vslot, int32_t* __restrict__ flag) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int got = *count;
-  if (got == expected) return;
-  *flag = 1;
-  for (int k = got > 0 ? got : 0; k < expected; ++k) {
-    iter[k] = 0;
-    iter_grp[k] = vslot[0];
-  }
-}
 }  // namespace
 
 void krylov_apply_A(double* Vb, int64_t vstride, const int32_t* iter_grp, int K, int jsrc, int jdst,
@@ -362,17 +379,11 @@ void krylov_apply_A(double* Vb, int64_t vstride, const int32_t* iter_grp, int K,
   apply_A_kernel<<<grid, 256, 0, st>>>(Vb, vstride, iter_grp, jsrc, jdst, rowptr, col, val, c, n);
 }
 
-void expect_count(const int32_t* count, int expected, int32_t* iter, int32_t* iter_grp,
-                  const int32_t* vslot, int32_t* flag, cudaStream_t st) {
-  expect_count_kernel<<<1, 32, 0, st>>>(count, expected, iter, iter_grp, vslot, flag);
-}
-
 void residual_check(SmallState ss, const RoundCols& rc, int K, int j, double gamma, double tol,
-                    int m_max, const int32_t* replay, const int32_t* iter_in, int32_t* iter_out,
-                    int32_t* iter_grp, int32_t* iter_count, cudaStream_t st) {
-  const size_t smem = sizeof(SmallShared);
-  residual_kernel<<<K, kSmallThreads, smem, st>>>(ss, rc, iter_in, j, gamma, tol, m_max, replay);
-  compact_kernel<<<1, 32, 0, st>>>(ss, rc.vslot, iter_in, K, iter_out, iter_grp, iter_count);
+                    int m_max, const int32_t* replay, const int32_t* iter_in, const CompactArgs& ca,
+                    cudaStream_t st) {
+  residual_kernel<<<K, kTeamThreads, sizeof(SmallShared<CtaTeam::kWorkers>), st>>>(
+      ss, rc, iter_in, j, gamma, tol, m_max, replay, ca);
 }
 
 void record_segments(const SmallState& ss, const RoundCols& rc, int K, int32_t* m_rec,
@@ -384,23 +395,18 @@ void record_segments(const SmallState& ss, const RoundCols& rc, int K, int32_t* 
 void output_coefficients(SmallState ss, const RoundCols& rc, int K, double gamma, double dt_out,
                          double* coef, int ldo, double* yend, cudaStream_t st, double tail_eps,
                          const double* pbound, int32_t* tcut) {
-  const size_t smem = sizeof(SmallShared);
-  coef_kernel<<<K, kSmallThreads, smem, st>>>(ss, rc, gamma, dt_out, coef, ldo, yend, tail_eps,
-                                              pbound, tcut);
+  coef_kernel<<<K, kTeamThreads, sizeof(SmallShared<CtaTeam::kWorkers>), st>>>(
+      ss, rc, gamma, dt_out, coef, ldo, yend, tail_eps, pbound, tcut);
 }
 
 void expm_batch(int batch, int m, const double* A, const double* h, double* E, cudaStream_t st) {
-  const size_t smem = sizeof(SmallShared);
-  expm_batch_kernel<<<batch, kSmallThreads, smem, st>>>(m, A, h, E);
+  expm_batch_kernel<<<batch, m <= 8 ? 64 : kSmallThreads, 0, st>>>(m, A, h, E);
 }
 
-size_t small_shared_bytes() { return sizeof(SmallShared); }
-
 void set_small_smem_limits() {
-  const int bytes = (int)sizeof(SmallShared);
+  const int bytes = (int)sizeof(SmallShared<CtaTeam::kWorkers>);
   cudaFuncSetAttribute(residual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   cudaFuncSetAttribute(coef_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(expm_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 }  // namespace matex

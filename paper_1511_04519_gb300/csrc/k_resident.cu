@@ -20,16 +20,31 @@ namespace matex {
 namespace {
 
 
-// Sum over the CTA, returned to every thread.  red: 32 doubles of shared memory.
-__device__ __forceinline__ double res_block_sum(double v, double* red) {
+// Norm of a vector whose squares' sums the threads hold, and its reciprocal (0
+// for a norm up to `least`), returned to every thread.  red: 32 doubles of
+// shared memory.  One warp adds the warps' sums and one thread takes the root
+// and the quotient: an FP64 instruction costs the CTA 64 clocks per four warps,
+// a division of all 512 threads 2,550 (measured).
+struct ResNorm {
+  double v, inv;
+};
+__device__ __forceinline__ ResNorm res_block_norm(double v, double least, double* red) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   __syncthreads();  // earlier readers of red are done
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  double s = 0.0;
-  const int nw = (int)(blockDim.x >> 5);
-  for (int i = 0; i < nw; ++i) s += red[i];
-  return s;
+  if (threadIdx.x < 32) {
+    const int nw = (int)(blockDim.x >> 5);
+    double s = (int)threadIdx.x < nw ? red[threadIdx.x] : 0.0;
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (threadIdx.x == 0) {
+      const double r = sqrt(s);
+      red[30] = r;
+      red[31] = r <= least ? 0.0 : 1.0 / r;
+    }
+  }
+  __syncthreads();
+  return ResNorm{red[30], red[31]};
 }
 
 
@@ -217,8 +232,9 @@ __device__ __forceinline__ void res_dots(const double* __restrict__ V, int64_t n
   }
 }
 
+template <class Team>
 __host__ __device__ constexpr size_t res_small_bytes() {
-  return (sizeof(SmallShared) + 15) & ~(size_t)15;
+  return (sizeof(SmallShared<Team::kWorkers>) + 15) & ~(size_t)15;
 }
 constexpr int kResHsh = 24;  // >= kMaxB, padded
 // solve kernel: the plan (16-byte aligned), then b, y, U
@@ -227,8 +243,9 @@ size_t res_solve_smem_bytes(int64_t n, const ResidentPlan& P) {
 }
 // round kernel: the small dense work, the dot products and reductions, then
 // as the solve kernel
+template <class Team>
 size_t res_smem_bytes(int64_t n, const ResidentPlan& P) {
-  return res_small_bytes() + sizeof(double) * ((size_t)kResHsh + 32) +
+  return res_small_bytes<Team>() + sizeof(double) * ((size_t)kResHsh + 32) +
          res_solve_smem_bytes(n, P);
 }
 
@@ -279,10 +296,11 @@ __device__ void res_inputs(const ResidentArgs& a, const ResSmem& ms, int q, doub
   for (int64_t i = tid; i < n; i += nt) W[i] = b[i];
 }
 
+template <class Team>
 __global__ void __launch_bounds__(kResidentThreads, 1) resident_round_kernel(ResidentArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SmallShared& sh = *reinterpret_cast<SmallShared*>(smem_raw);
-  double* hsh = reinterpret_cast<double*>(smem_raw + res_small_bytes());
+  SmallShared<Team::kWorkers>& sh = *reinterpret_cast<SmallShared<Team::kWorkers>*>(smem_raw);
+  double* hsh = reinterpret_cast<double*>(smem_raw + res_small_bytes<Team>());
   int* stflag = reinterpret_cast<int*>(hsh + kResHsh - 1);  // past the kMaxB dot products
   double* red = hsh + kResHsh;
   unsigned char* pl = reinterpret_cast<unsigned char*>(red + 32);  // 16-byte aligned
@@ -333,7 +351,8 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_round_kernel(Res
       acc = fma(v, v, acc);
     }
   }
-  const double beta = sqrt(res_block_sum(acc, red));
+  const ResNorm nb = res_block_norm(acc, 1e-300, red);
+  const double beta = nb.v;
   double* Ht = ss.Ht + (int64_t)q * kMaxB * kMaxM;
   for (int e = tid; e < kMaxB * kMaxM; e += nt) Ht[e] = 0.0;
   const bool quiet = beta <= 1e-300;
@@ -341,11 +360,10 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_round_kernel(Res
     ss.beta[q] = beta;
     ss.m[q] = 0;
     ss.status[q] = quiet ? 4 : 0;
-    ss.scale[q] = quiet ? 0.0 : 1.0 / beta;
+    ss.scale[q] = nb.inv;
   }
   if (!quiet) {
-    const double sc = 1.0 / beta;
-    for (int64_t i = tid; i < n; i += nt) V[i] = b[i] * sc;
+    for (int64_t i = tid; i < n; i += nt) V[i] = b[i] * nb.inv;
     for (int j = 0; j < a.m_max; ++j) {
       // w = X1^{-1} C v_j (Alg. 1 with X2 = C)
       const double* __restrict__ vj = V + (int64_t)j * n;
@@ -367,19 +385,21 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_round_kernel(Res
       }
       double a2 = 0.0;
       for (int64_t i = tid; i < n; i += nt) a2 = fma(b[i], b[i], a2);
-      const double nrm = sqrt(res_block_sum(a2, red));
-      const double sc2 = nrm > 0.0 ? 1.0 / nrm : 0.0;
+      const ResNorm nw = res_block_norm(a2, 0.0, red);
+      const double nrm = nw.v, sc2 = nw.inv;
       if (tid == 0) {
         Ht[(j + 1) * kMaxM + j] = nrm;
         ss.scale[q] = sc2;
       }
       double* __restrict__ vn = V + (int64_t)(j + 1) * n;
       for (int64_t i = tid; i < n; i += nt) vn[i] = b[i] * sc2;
-      // the residual test (small dense work) by warp 0 alone: warp barriers
-      // instead of CTA barriers between its many short steps
+      // the residual test (small dense work) by the first warps alone: their
+      // barriers instead of the CTA's between its many short steps, one
+      // exponential per warp, the coefficients' among them
       __syncthreads();
-      if (tid < 32) {
-        const int st = residual_column<WarpGroup>(ss, rc, q, j, a.gamma, a.tol, a.m_max, a.replay, sh);
+      if (tid < 32 * Team::kWorkers) {
+        const int st = residual_column<Team>(ss, rc, q, j, a.gamma, a.tol, a.m_max, a.replay,
+                                             rc.nout[q] > 1 ? a.dt_out : 0.0, sh);
         if (tid == 0) *stflag = st;
       }
       __syncthreads();
@@ -387,9 +407,8 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_round_kernel(Res
     }
   }
   __syncthreads();
-  if (tid < 32)
-    coef_column<WarpGroup>(ss, rc, q, a.gamma, a.dt_out, a.coef, a.ldo, a.yend, 0.0, nullptr, nullptr,
-                           sh);
+  if (tid < 32 * Team::kWorkers)
+    coef_column<Team>(ss, rc, q, a.gamma, a.dt_out, a.coef, a.ldo, a.yend, 0.0, nullptr, nullptr, sh);
   __syncthreads();
   // state at the segment's end: x = z + L z' - w + V y(L)
   const int m = ss.m[q];
@@ -464,32 +483,51 @@ bool resident_fits(int64_t n, const ResidentPlan& P) {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return n > 0 && n <= kResidentMaxN && res_smem_bytes(n, P) <= (size_t)optin;
+  return n > 0 && n <= kResidentMaxN && res_smem_bytes<WarpSolo>(n, P) <= (size_t)optin;
 }
+
+namespace {
+// three exponentials at once where their work areas fit beside the rest
+bool res_team(int64_t n, const ResidentPlan& P) {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return res_smem_bytes<WarpTeam>(n, P) <= (size_t)optin;
+}
+}  // namespace
 
 bool resident_set_limits(int64_t n, const ResidentPlan& P) {
   // the kernels' limits only grow: contexts of several sizes share them
-  static size_t done = 0;
-  const size_t bytes = res_smem_bytes(n, P);
-  if (bytes <= done) return true;
-  const bool ok =
-      cudaFuncSetAttribute(resident_round_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)bytes) == cudaSuccess &&
-      cudaFuncSetAttribute(resident_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)res_solve_smem_bytes(n, P)) == cudaSuccess &&
-      cudaFuncSetAttribute(resident_inputs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)res_solve_smem_bytes(n, P)) == cudaSuccess;
-  if (!ok) {
-    cudaGetLastError();
-    return false;
+  static size_t done[2] = {0, 0};
+  const bool team = res_team(n, P);
+  const size_t bytes = team ? res_smem_bytes<WarpTeam>(n, P) : res_smem_bytes<WarpSolo>(n, P);
+  const size_t solve = res_solve_smem_bytes(n, P);
+  bool ok = true;
+  if (bytes > done[team]) {
+    ok = (team ? cudaFuncSetAttribute(resident_round_kernel<WarpTeam>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
+               : cudaFuncSetAttribute(resident_round_kernel<WarpSolo>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) == cudaSuccess;
+    if (ok) done[team] = bytes;
   }
-  done = bytes;
-  return true;
+  static size_t solve_done = 0;
+  if (ok && solve > solve_done) {
+    ok = cudaFuncSetAttribute(resident_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)solve) == cudaSuccess &&
+         cudaFuncSetAttribute(resident_inputs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)solve) == cudaSuccess;
+    if (ok) solve_done = solve;
+  }
+  if (!ok) cudaGetLastError();
+  return ok;
 }
 
 void resident_round(const ResidentArgs& a, int K, cudaStream_t st) {
   if (K <= 0) return;
-  resident_round_kernel<<<K, kResidentThreads, res_smem_bytes(a.n, a.plan), st>>>(a);
+  if (res_team(a.n, a.plan))
+    resident_round_kernel<WarpTeam><<<K, kResidentThreads, res_smem_bytes<WarpTeam>(a.n, a.plan), st>>>(a);
+  else
+    resident_round_kernel<WarpSolo><<<K, kResidentThreads, res_smem_bytes<WarpSolo>(a.n, a.plan), st>>>(a);
 }
 
 void resident_inputs(const ResidentArgs& a, int K, cudaStream_t st) {

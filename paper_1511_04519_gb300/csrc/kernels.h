@@ -216,29 +216,36 @@ struct SmallState {
   double rscale = 1.0;  // factor on h_{m+1,m} in the residual: 1, 1/gamma, gamma
 };
 
+// Where the kernels that decide the columns' status put the list of those
+// still iterating: columns in order (iter_out), their basis slots (slots of the
+// round's columns; iter_grp) and their number.  arrived: a counter, zero
+// between launches (the last CTA of a launch makes the list).  expected >= 0, in
+// a recorded (graph) run: the number its launches were sized for; another one
+// raises *flag and the entries from it up to expected point at column 0 of the
+// round, so that the rest of the replay (whose result is then discarded) stays
+// in range.
+struct CompactArgs {
+  const int32_t* slots;
+  int32_t *iter_out, *iter_grp, *count, *arrived, *flag;
+  int expected;
+};
 // finish the start vector: beta = sqrt(sum partials), scale = 1/beta, status;
-// writes the list of non-quiescent columns and its count
-void start_finish(const double* partials, int nchunks, int K, SmallState ss, const int32_t* groups,
-                  int32_t* iter_out, int32_t* iter_grp, int32_t* iter_count, cudaStream_t st);
+// lists the non-quiescent columns
+void start_finish(const double* partials, int nchunks, int K, SmallState ss, const CompactArgs& ca,
+                  cudaStream_t st);
 // reduce dot partials into hbuf (and accumulate into Ht column j when acc != 0)
 void reduce_dots(const double* partials, int nchunks, int K, int nb, const int32_t* iter,
                  SmallState ss, int j, int mode, cudaStream_t st);
-// residual test after step j (m = j+1): decides status per column; writes
-// the compacted list of still-iterating columns and its count
-// Guard of a recorded (graph) run: when *count differs from the count the
-// recorded launches were sized for, raise *flag and point the entries
-// [*count, expected) of iter / iter_grp at column 0 of the round, so that the
-// rest of the replay (whose result is then discarded) stays in range.
-void expect_count(const int32_t* count, int expected, int32_t* iter, int32_t* iter_grp,
-                  const int32_t* vslot, int32_t* flag, cudaStream_t st);
 // w = A v = -C^{-1} G v for the standard Krylov space: column q of the batch
 // reads slot `jsrc` of its basis and writes slot `jdst` (G in CSR, permuted).
 void krylov_apply_A(double* Vb, int64_t vstride, const int32_t* iter_grp, int K, int jsrc, int jdst,
                     const int64_t* rowptr, const int32_t* col, const double* val, const double* c,
                     int64_t n, cudaStream_t st);
+// residual test after step j (m = j+1) of the K columns of iter_in: decides
+// their status, lists those still iterating
 void residual_check(SmallState ss, const RoundCols& rc, int K, int j, double gamma, double tol,
-                    int m_max, const int32_t* replay, const int32_t* iter_in, int32_t* iter_out,
-                    int32_t* iter_grp, int32_t* iter_count, cudaStream_t st);
+                    int m_max, const int32_t* replay, const int32_t* iter_in, const CompactArgs& ca,
+                    cudaStream_t st);
 // record m and status of the round's columns at their global segment ids
 void record_segments(const SmallState& ss, const RoundCols& rc, int K, int32_t* m_rec,
                      int32_t* st_rec, cudaStream_t st);
@@ -257,7 +264,6 @@ void output_coefficients(SmallState ss, const RoundCols& rc, int K, double gamma
 // z + h z' - w for every h in [0, L] (a NaN anywhere makes the bound NaN)
 void p_bound(const double* Z, const double* Zp, const double* W, int64_t gstride,
              const RoundCols& rc, int K, int64_t n, double* pbound, cudaStream_t st);
-size_t small_shared_bytes();
 void set_small_smem_limits();
 // batched expm for the public test entry point
 void expm_batch(int batch, int m, const double* A, const double* h, double* E, cudaStream_t st);

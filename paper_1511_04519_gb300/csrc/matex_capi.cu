@@ -1547,9 +1547,9 @@ bool ensure_g_csr(matex_ctx* c) {
 // One pass of the run (everything up to the output permutation) on c->st.
 // Plain (capture = false): the host reads every active-column count from the
 // device and appends it to kit_trace.  Recording (capture = true): the stream
-// is being captured into a CUDA graph; each count is taken from kit_trace and
-// followed by a guard kernel that raises the divergence flag (and keeps every
-// index in range) if the device count differs when the graph is replayed.
+// is being captured into a CUDA graph; each count is taken from kit_trace, and
+// the kernel that makes it on the device raises the divergence flag (and keeps
+// every index in range) if it differs when the graph is replayed.
 matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
   cudaStream_t st = c->st;
   const int64_t n = c->n;
@@ -1559,7 +1559,13 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
   int64_t solve_cols_total = 0;
   int e;
   size_t tpos = 0;
-  auto count = [&](int* out, int32_t* iter_now, const int32_t* vslot) -> matex_status {
+  // the next active-column count: read back (plain run), or as recorded and
+  // checked on the device by the kernel that makes it (capture)
+  auto next_list = [&](int32_t* iter_out, const int32_t* vslot) {
+    return CompactArgs{vslot, iter_out, c->iter_grp, c->d_count, c->d_count + 3, c->d_count + 2,
+                       capture && tpos < c->kit_trace.size() ? c->kit_trace[tpos] : -1};
+  };
+  auto count = [&](int* out) -> matex_status {
     if (!capture) {
       const matex_status rs = read_count(c, out);
       if (rs == MATEX_OK) c->kit_trace.push_back(*out);
@@ -1567,8 +1573,6 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
     }
     if (tpos >= c->kit_trace.size()) return fail(c, MATEX_ERR_STATE, "count trace too short");
     *out = c->kit_trace[tpos++];
-    expect_count(c->d_count, *out, iter_now, c->iter_grp, vslot, c->d_count + 2, st);
-    launches++;
     return MATEX_OK;
   };
   cudaMemsetAsync(c->d_count, 0, 4 * sizeof(int32_t), st);
@@ -1752,13 +1756,13 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
                  c->nchunks, st);
     prof_end(c, e, P_OTHER, 1, 4.0 * nd * K, 32.0 * nd * K);
     e = prof_begin(c);
-    start_finish(c->partials, c->nchunks, K, c->ss, rc.vslot, c->iterA, c->iter_grp, c->d_count, st);
+    start_finish(c->partials, c->nchunks, K, c->ss, next_list(c->iterA, rc.vslot), st);
     prof_end(c, e, P_SMALL, 1, 0.0, 0.0);
     launches += 2;
     int kit = 0;
     int32_t* iter = c->iterA;
     int32_t* iter_next = c->iterB;
-    if ((s = count(&kit, iter, rc.vslot)) != MATEX_OK) return s;
+    if ((s = count(&kit)) != MATEX_OK) return s;
     if (kit > 0) {
       e = prof_begin(c);
       basis_scale(c->Vb, vstride, rc.vslot, iter, kit, 0, c->ss.scale, n, st);
@@ -1807,12 +1811,12 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
       basis_scale(c->Vb, vstride, rc.vslot, iter, kit, j + 1, c->ss.scale, n, st);
       prof_end(c, e, P_GS, 9, (8.0 * j + 11.0) * nd * kit, (4.0 * j + 13.0) * 8.0 * nd * kit);
       e = prof_begin(c);
-      residual_check(c->ss, rc, kit, j, c->gamma, c->tol, c->m_max, c->replay_d, iter, iter_next,
-                     c->iter_grp, c->d_count, st);
-      prof_end(c, e, P_SMALL, 2, 0.0, 0.0);
-      launches += 11;
+      residual_check(c->ss, rc, kit, j, c->gamma, c->tol, c->m_max, c->replay_d, iter,
+                     next_list(iter_next, rc.vslot), st);
+      prof_end(c, e, P_SMALL, 1, 0.0, 0.0);
+      launches += 10;
       std::swap(iter, iter_next);
-      if ((s = count(&kit, iter, rc.vslot)) != MATEX_OK) return s;
+      if ((s = count(&kit)) != MATEX_OK) return s;
     }
     if (c->opts.tape == 1) tape_small(c->ss, rc, K, c->THt, c->Tbeta, st);
     e = prof_begin(c);
@@ -2093,8 +2097,8 @@ matex_status reverse_round(matex_ctx* c, const Round& r, int qa, int K, const in
 // (the block's groups) from the checkpoint of window w, keeping each
 // segment's basis, solve outputs, z', Hessenberg and norm in window-tape slot
 // i * Kb + (column - qa[i]).  The Krylov dimensions are the run's (replay of
-// m_rec); the active-column counts are known on the host, and guard kernels
-// check them on the device as in a graph replay (a mismatch raises the
+// m_rec); the active-column counts are known on the host and checked on the
+// device as in a graph replay (a mismatch raises the
 // divergence flag and keeps every index in range).
 matex_status recompute_window(matex_ctx* c, int w, int r0, int r1, const std::vector<int>& qa,
                               const std::vector<int>& qb, int g0, int g1,
@@ -2134,8 +2138,6 @@ matex_status recompute_window(matex_ctx* c, int w, int r0, int r1, const std::ve
     scatter_cols(c->Y, c->ldy, K, c->Wb, n, rc.group, nullptr, n, st);
     krylov_start(c->Vb, vstride, c->Xb, c->Zb, c->Wb, n, rc.group, rc.vslot, K, n, c->partials,
                  c->nchunks, st);
-    start_finish(c->partials, c->nchunks, K, c->ss, rc.vslot, c->iterA, c->iter_grp, c->d_count,
-                 st);
     int32_t* iter = c->iterA;
     int32_t* iter_next = c->iterB;
     auto active = [&](int above) {
@@ -2143,8 +2145,11 @@ matex_status recompute_window(matex_ctx* c, int w, int r0, int r1, const std::ve
       for (int q = 0; q < K; ++q) k += mrec[b0 + q] > above ? 1 : 0;
       return k;
     };
+    auto next_list = [&](int32_t* out, int expected) {
+      return CompactArgs{rc.vslot, out, c->iter_grp, c->d_count, c->d_count + 3, c->d_count + 2, expected};
+    };
     int kit = active(0);
-    expect_count(c->d_count, kit, iter, c->iter_grp, rc.vslot, c->d_count + 2, st);
+    start_finish(c->partials, c->nchunks, K, c->ss, next_list(iter, kit), st);
     if (kit > 0) basis_scale(c->Vb, vstride, rc.vslot, iter, kit, 0, c->ss.scale, n, st);
     for (int j = 0; j < c->m_max && kit > 0; ++j) {
       gather_cols(c->Y, c->ldy, kit, c->Vb + (int64_t)j * n, vstride, c->iter_grp, c->c_perm,
@@ -2164,11 +2169,11 @@ matex_status recompute_window(matex_ctx* c, int w, int r0, int r1, const std::ve
                  st);
       reduce_dots(c->partials, c->nchunks, kit, 1, iter, c->ss, j, 2, st);
       basis_scale(c->Vb, vstride, rc.vslot, iter, kit, j + 1, c->ss.scale, n, st);
-      residual_check(c->ss, rc, kit, j, c->gamma, c->tol, c->m_max, c->m_rec, iter, iter_next,
-                     c->iter_grp, c->d_count, st);
+      const int left = active(j + 1);
+      residual_check(c->ss, rc, kit, j, c->gamma, c->tol, c->m_max, c->m_rec, iter,
+                     next_list(iter_next, left), st);
       std::swap(iter, iter_next);
-      kit = active(j + 1);
-      expect_count(c->d_count, kit, iter, c->iter_grp, rc.vslot, c->d_count + 2, st);
+      kit = left;
     }
     tape_small(c->ss, rc, K, c->THt, c->Tbeta, st);
     output_coefficients(c->ss, rc, K, c->gamma, c->dt_out, c->coef, c->n_times, c->yend, st);
