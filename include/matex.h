@@ -101,12 +101,11 @@ typedef struct matex_opts {
                               memory) */
   int32_t tape_block;      /* tape = 2: groups recomputed together (columns of the recompute
                               and reverse launches); 0 (default): chosen at setup */
-  int32_t recombine;       /* V y of the recombination (Eq. 6 at the outputs): 0 (default) on
-                              the tensor cores where it pays (exact runs, rounds of 16 to
-                              kdim_cap basis vectors), as an error-free decomposition of the
-                              FP64 operands into 6-bit bf16 slices whose products the FP32
-                              accumulators hold exactly (error of the order of an FP64 dot
-                              product); 1: FP64 FMAs only */
+  int32_t recombine;       /* the recombination (Eq. 6 at the outputs): 0 (default) on the
+                              tensor cores where enough terms meet in an output, as an
+                              error-free split of the FP64 operands into seven 8-bit digits
+                              whose products the FP32 accumulators hold exactly (error no
+                              larger than an FP64 dot product's); 1: FP64 FMAs only */
   int32_t decompose;       /* 0 (default): the groups as given (Sec. 3.1's bump groups);
                               1: every group's input is split further into single ramps: on
                               [0, T] a source is its value at t = 0 plus, at each of its
@@ -180,7 +179,9 @@ typedef struct matex_stats {
   int32_t tape_block;      /*   block as set up (0 otherwise) */
   int64_t tape_bytes;      /* device bytes of the adjoint's tape (tape 1) or of its checkpoints,
                               window tape and reverse work buffers (tape 2) */
-  int32_t tc_rounds;       /* segment rounds of the last run whose V y ran on the tensor cores */
+  int32_t tc_rounds;       /* dense segment rounds of the last exact run on the tensor cores: at
+                              least 16 basis vectors, whose columns hold at least a quarter of
+                              the round's outputs (sparser rounds may run there too) */
   int32_t resident;        /* 1: the segment rounds run as resident rounds (opts.resident) */
   int32_t tc_solve_supernodes;  /* supernodes at least tc_min_width wide whose solve products
                                    can run on the tensor cores (0: none or tc_solve off) */

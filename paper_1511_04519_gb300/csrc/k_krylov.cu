@@ -28,8 +28,9 @@ __global__ void input_rhs_kernel(double* __restrict__ Y, int ldy, int K, RoundCo
 
 __global__ void advance_z_kernel(double* __restrict__ Z, const double* __restrict__ Zp,
                                  const double* __restrict__ X, int64_t gstride, RoundCols rc,
-                                 int64_t n) {
+                                 int64_t n, double* __restrict__ pbound) {
   const int q = blockIdx.y;
+  if (blockIdx.x == 0 && threadIdx.x < 2) pbound[2 * q + threadIdx.x] = 0.0;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t g = rc.group[q];
@@ -66,9 +67,11 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 
 __global__ void __launch_bounds__(kRedThreads)
 krylov_start_kernel(double* __restrict__ Vb, int64_t vstride, const double* __restrict__ X,
-                    const double* __restrict__ Z, const double* __restrict__ W, int64_t gstride,
-                    const int32_t* __restrict__ groups, const int32_t* __restrict__ vslots,
-                    int64_t n, double* __restrict__ partials, int nchunks) {
+                    const double* __restrict__ Z, const double* __restrict__ Zp,
+                    const double* __restrict__ W, unsigned long long* __restrict__ pbound,
+                    int64_t gstride, const int32_t* __restrict__ groups,
+                    const int32_t* __restrict__ vslots, int64_t n, double* __restrict__ partials,
+                    int nchunks) {
   __shared__ double red[32];
   const int q = blockIdx.y;
   const int64_t g = groups[q];
@@ -76,10 +79,25 @@ krylov_start_kernel(double* __restrict__ Vb, int64_t vstride, const double* __re
   const int64_t b = (int64_t)blockIdx.x * kChunk;
   const int64_t e = min(n, b + kChunk);
   double acc = 0.0;
+  // |w - z| and |z'| are >= 0 (or NaN without its sign bit): their bit patterns
+  // order like the values, a NaN above +inf
+  unsigned long long pa = 0, pb = 0;
+  constexpr unsigned long long kAbs = 0x7fffffffffffffffull;
   for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) {
-    const double v = X[g * gstride + i] + (W[g * gstride + i] - Z[g * gstride + i]);
+    const double wz = W[g * gstride + i] - Z[g * gstride + i];
+    const double v = X[g * gstride + i] + wz;
     Vb[vs * vstride + i] = v;
     acc = fma(v, v, acc);
+    pa = max(pa, (unsigned long long)__double_as_longlong(wz) & kAbs);
+    pb = max(pb, (unsigned long long)__double_as_longlong(Zp[g * gstride + i]) & kAbs);
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    pa = max(pa, __shfl_xor_sync(0xffffffffu, pa, off));
+    pb = max(pb, __shfl_xor_sync(0xffffffffu, pb, off));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(pbound + 2 * q, pa);
+    atomicMax(pbound + 2 * q + 1, pb);
   }
   const double s = block_sum(acc, red);
   if (threadIdx.x == 0) partials[(int64_t)q * nchunks + blockIdx.x] = s;
@@ -305,10 +323,10 @@ void build_input_rhs(double* Y, int ldy, int K, const RoundCols& rc, const Sourc
 }
 
 void advance_z(double* Z, const double* Zp, const double* X, int64_t gstride, const RoundCols& rc,
-               int K, int64_t n, cudaStream_t st) {
+               int K, int64_t n, double* pbound, cudaStream_t st) {
   if (K <= 0) return;
   dim3 grid((unsigned)((n + 255) / 256), (unsigned)K);
-  advance_z_kernel<<<grid, 256, 0, st>>>(Z, Zp, X, gstride, rc, n);
+  advance_z_kernel<<<grid, 256, 0, st>>>(Z, Zp, X, gstride, rc, n, pbound);
 }
 
 void build_initial_rhs(double* Y, int ldy, int K, const SourceTable& src, const int32_t* groups,
@@ -317,12 +335,13 @@ void build_initial_rhs(double* Y, int ldy, int K, const SourceTable& src, const 
   initial_rhs_kernel<<<(K + 127) / 128, 128, 0, st>>>(Y, ldy, K, src, groups);
 }
 
-void krylov_start(double* Vbase, int64_t vstride, const double* X, const double* Z, const double* W,
-                  int64_t gstride, const int32_t* groups, const int32_t* vslots, int K, int64_t n,
+void krylov_start(double* Vbase, int64_t vstride, const double* X, const double* Z, const double* Zp,
+                  const double* W, double* pbound, int64_t gstride, const int32_t* groups, const int32_t* vslots, int K, int64_t n,
                   double* partials, int nchunks, cudaStream_t st) {
   dim3 grid((unsigned)nchunks, (unsigned)K);
-  krylov_start_kernel<<<grid, kRedThreads, 0, st>>>(Vbase, vstride, X, Z, W, gstride, groups,
-                                                    vslots, n, partials, nchunks);
+  krylov_start_kernel<<<grid, kRedThreads, 0, st>>>(
+      Vbase, vstride, X, Z, Zp, W, reinterpret_cast<unsigned long long*>(pbound), gstride, groups,
+      vslots, n, partials, nchunks);
 }
 
 void basis_dots(const double* Vbase, int64_t vstride, const int32_t* groups, const int32_t* iter,

@@ -129,43 +129,6 @@ recombine_kernel(double* __restrict__ Xp, int64_t n, const double* __restrict__ 
     }
 }
 
-// Per column, the largest |z - w| and |z'| of its group over a chunk of nodes,
-// folded into pbound by an atomic max.  Both are >= 0 (or NaN with the sign
-// bit clear), so their bit patterns order like the values and a NaN, whose
-// pattern is above +inf's, is kept.
-constexpr int kPbThreads = 256;
-constexpr int kPbPer = 8;  // nodes per thread
-
-__global__ void __launch_bounds__(kPbThreads)
-p_bound_kernel(const double* __restrict__ Z, const double* __restrict__ Zp,
-               const double* __restrict__ W, int64_t gstride, RoundCols rc, int64_t n,
-               unsigned long long* __restrict__ pbound) {
-  const int q = blockIdx.y;
-  const int64_t g = rc.group[q];
-  const double* __restrict__ z = Z + g * gstride;
-  const double* __restrict__ zp = Zp + g * gstride;
-  const double* __restrict__ w = W + g * gstride;
-  unsigned long long a = 0, b = 0;
-  const int64_t base = (int64_t)blockIdx.x * kPbThreads * kPbPer + threadIdx.x;
-#pragma unroll
-  for (int k = 0; k < kPbPer; ++k) {
-    const int64_t i = base + (int64_t)k * kPbThreads;
-    if (i < n) {
-      a = max(a, (unsigned long long)__double_as_longlong(fabs(z[i] - w[i])));
-      b = max(b, (unsigned long long)__double_as_longlong(fabs(zp[i])));
-    }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    a = max(a, __shfl_xor_sync(0xffffffffu, a, off));
-    b = max(b, __shfl_xor_sync(0xffffffffu, b, off));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(pbound + 2 * q, a);
-    atomicMax(pbound + 2 * q + 1, b);
-  }
-}
-
 __global__ void next_state_kernel(double* __restrict__ X, const double* __restrict__ Vb,
                                   int64_t vstride, const double* __restrict__ Z,
                                   const double* __restrict__ Zp, const double* __restrict__ W,
@@ -181,47 +144,6 @@ __global__ void next_state_kernel(double* __restrict__ X, const double* __restri
   const double* __restrict__ base = Vb + (int64_t)rc.vslot[q] * vstride + i;
   for (int j = 0; j < m; ++j) s = fma(base[(int64_t)j * n], yend[q * kMaxM + j], s);
   X[g * gstride + i] = s;
-}
-
-// The -P terms of a round alone, X[o] += sum over the columns whose segment
-// holds o of z + (t_o - l_j) z' - w = (z - w - l_j z') + t_o z'.  Which
-// columns hold o changes only where a column's output range starts or ends:
-// one thread per node sweeps the outputs in order, keeping the two running
-// sums A = sum (z - w - l_j z') and B = sum z' of the columns holding o and
-// updating them at those events (sorted by output: ev_o; ev_q = q + 1 when
-// column q enters, -(q + 1) when it leaves).  Each column's z, z', w are read
-// once per node, not once per output tile.
-__global__ void __launch_bounds__(128)
-recombine_p_kernel(double* __restrict__ Xp, int64_t n, const double* __restrict__ Z,
-                   const double* __restrict__ Zp, const double* __restrict__ W, int64_t gstride,
-                   RoundCols rc, const int32_t* __restrict__ ev_o, const int32_t* __restrict__ ev_q,
-                   int nev, int o_begin, int o_end, double dt_out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || (rc.abort && *rc.abort)) return;
-  double A = 0.0, B = 0.0;
-  int active = 0, e = 0;
-  for (int o = o_begin; o < o_end; ++o) {
-    for (; e < nev && ev_o[e] <= o; ++e) {
-      const int qs = ev_q[e];
-      const int q = (qs > 0 ? qs : -qs) - 1;
-      const int64_t g = rc.group[q];
-      const double zp = Zp[g * gstride + i];
-      const double a = fma(-rc.l0[q], zp, Z[g * gstride + i] - W[g * gstride + i]);
-      if (qs > 0) {
-        A += a;
-        B += zp;
-        active++;
-      } else {
-        A -= a;
-        B -= zp;
-        active--;
-      }
-    }
-    if (active > 0) {
-      double* x = Xp + (int64_t)o * n + i;
-      *x += fma((double)o * dt_out, B, A);
-    }
-  }
 }
 
 // Checkpoint of column q: CK[q] = {X[group q], Z[group q]} (save), or back (restore).
@@ -282,30 +204,12 @@ void recombine(double* Xp, int64_t n, int n_times, const double* Vbase, int64_t 
                                                   coef, ldo, K, obeg_min, dt_out, tcut);
 }
 
-void p_bound(const double* Z, const double* Zp, const double* W, int64_t gstride,
-             const RoundCols& rc, int K, int64_t n, double* pbound, cudaStream_t st) {
-  if (K <= 0) return;
-  cudaMemsetAsync(pbound, 0, sizeof(double) * 2 * (size_t)K, st);
-  const int64_t per = (int64_t)kPbThreads * kPbPer;
-  dim3 grid((unsigned)((n + per - 1) / per), (unsigned)K);
-  p_bound_kernel<<<grid, kPbThreads, 0, st>>>(Z, Zp, W, gstride, rc, n,
-                                              reinterpret_cast<unsigned long long*>(pbound));
-}
-
 void next_state(double* X, const double* Vbase, int64_t vstride, const double* Z, const double* Zp,
                 const double* W, int64_t gstride, const RoundCols& rc, const int32_t* mcol,
                 const double* yend, int K, int64_t n, cudaStream_t st) {
   if (K <= 0) return;
   dim3 grid((unsigned)((n + 255) / 256), (unsigned)K);
   next_state_kernel<<<grid, 256, 0, st>>>(X, Vbase, vstride, Z, Zp, W, gstride, rc, mcol, yend, n);
-}
-
-void recombine_p(double* Xp, int64_t n, const double* Z, const double* Zp, const double* W,
-                 int64_t gstride, const RoundCols& rc, const int32_t* ev_o, const int32_t* ev_q,
-                 int nev, int o_begin, int o_end, double dt_out, cudaStream_t st) {
-  if (nev <= 0 || o_end <= o_begin) return;
-  recombine_p_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(Xp, n, Z, Zp, W, gstride, rc, ev_o,
-                                                                  ev_q, nev, o_begin, o_end, dt_out);
 }
 
 void checkpoint_states(double* CK, double* X, double* Z, const int32_t* groups, int K, int64_t n,

@@ -178,16 +178,20 @@ void tr_store(double* x, const double* Y, int ldy, double* Xp, int64_t row, int6
 // Y[:, q] = B_k (u_k(l0+L) - u_k(l0)) / L, the input slope on the segment (Y zeroed here)
 void build_input_rhs(double* Y, int ldy, int K, const RoundCols& rc, const SourceTable& src,
                      int64_t n, cudaStream_t st);
-// z_k = x_k for a group's first segment, else z_k += lprev * z'_k
+// z_k = x_k for a group's first segment, else z_k += lprev * z'_k; pbound[2q],
+// pbound[2q + 1] = 0
 void advance_z(double* Z, const double* Zp, const double* X, int64_t gstride, const RoundCols& rc,
-               int K, int64_t n, cudaStream_t st);
+               int K, int64_t n, double* pbound, cudaStream_t st);
 // Y[:, q] = B_k u_k(t) for t = 0 per group (initial states)
 void build_initial_rhs(double* Y, int ldy, int K, const SourceTable& src, const int32_t* groups,
                        int64_t n, cudaStream_t st);
 
-// Krylov start: v = x - z + w written to V[vslot][0]; partial sums of |v|^2
-void krylov_start(double* Vbase, int64_t vstride, const double* X, const double* Z,
-                  const double* W, int64_t gstride, const int32_t* groups, const int32_t* vslots,
+// Krylov start: v = x - z + w written to V[vslot][0]; partial sums of |v|^2;
+// pbound[2q] = max_i |z_i - w_i| and pbound[2q + 1] = max_i |z'_i| (zero before),
+// so that pbound[2q] + L pbound[2q + 1] bounds the column's -P term z + h z' - w
+// for every h in [0, L] (a NaN anywhere makes the bound NaN)
+void krylov_start(double* Vbase, int64_t vstride, const double* X, const double* Z, const double* Zp,
+                  const double* W, double* pbound, int64_t gstride, const int32_t* groups, const int32_t* vslots,
                   int K, int64_t n, double* partials, int nchunks, cudaStream_t st);
 
 // Partial dot products of basis slot wslot (w) with slots first..first+nb-1
@@ -259,11 +263,6 @@ void output_coefficients(SmallState ss, const RoundCols& rc, int K, double gamma
                          double* coef, int ldo, double* yend, cudaStream_t st,
                          double tail_eps = 0.0, const double* pbound = nullptr,
                          int32_t* tcut = nullptr);
-// pbound[2q] = max_i |z_i - w_i| and pbound[2q+1] = max_i |z'_i| over the
-// column's group, so that pbound[2q] + L pbound[2q+1] bounds its -P term
-// z + h z' - w for every h in [0, L] (a NaN anywhere makes the bound NaN)
-void p_bound(const double* Z, const double* Zp, const double* W, int64_t gstride,
-             const RoundCols& rc, int K, int64_t n, double* pbound, cudaStream_t st);
 void set_small_smem_limits();
 // batched expm for the public test entry point
 void expm_batch(int batch, int m, const double* A, const double* h, double* E, cudaStream_t st);
@@ -282,39 +281,43 @@ void recombine(double* Xp, int64_t n, int n_times, const double* Vbase, int64_t 
 void next_state(double* X, const double* Vbase, int64_t vstride, const double* Z, const double* Zp,
                 const double* W, int64_t gstride, const RoundCols& rc, const int32_t* mcol,
                 const double* yend, int K, int64_t n, cudaStream_t st);
-// Tensor-core recombination of the V y part (k_recombine_tc.cu): error-free
-// 6-bit slices of V (per node) and of the coefficients (per output) in bf16,
-// tcgen05 MMAs into FP32 accumulators that stay exact integers, exact
-// integer combination, FP64 result added into Xp.  Scratch of a context,
-// sized at setup for rounds of up to kdim_cap basis vectors.
-constexpr int kTcMaxKdim = 2048;  // basis vectors of one round the scratch may be sized for
-constexpr int kTcMinKdim = 16;    // below this the FP64 kernel is cheaper
-struct TcScratch {
-  void* slices = nullptr;       // V and coefficient slices in the MMA tile layout
-  int64_t* kmap = nullptr;      // [kdim_cap] basis vector -> offset in Vbase
-  int32_t* kq = nullptr;        // [kdim_cap] basis vector -> (column << 5) | index
-  double* rowscale = nullptr;   // [n] power-of-two scale of each node's basis values
-  double* colscale = nullptr;   // [output tiles x 48] scale of each output's coefficients
-  int32_t* err = nullptr;       // raised when a bounded wait of the MMA kernel gives up
-  int kdim_cap = 0;
+// Recombination on the tensor cores (k_recombine_mma.cu).  One term k of a
+// round's contraction: vector at offset off (of the bases, or of a group's z'
+// and z - w), column q, j: its basis index, kMaxM for z' (coefficient h) and
+// kMaxM + 1 for z - w (coefficient 1); outputs [ob, oe); the vector is taken
+// times 2^-sc, its coefficients times 2^sc.
+struct RmK {
+  int64_t off;
+  int32_t q, j, ob, oe, sc, pad;
 };
-size_t tc_slices_bytes(int64_t n, int kdim, int nouts);
-void tc_set_limits();
-// Xp[o][i] += sum over the round's columns q and j < mcol[q] of V_q[j][i] y_q(o)[j]
-// for o in [obeg_min, oend_max) (the columns' own output ranges); kdim = sum
-// of mcol.  Returns the number of kernels launched.
-int recombine_tc(double* Xp, int64_t n, const double* Vbase, int64_t vstride, const RoundCols& rc,
-                 const int32_t* mcol, const double* coef, int ldo, int K, int kdim, int obeg_min,
-                 int oend_max, const TcScratch& ts, cudaStream_t st);
-
-// The -P terms z + h z' - w of a round's columns at their outputs, added into
-// Xp by one sweep over the outputs per node; events ev_o / ev_q (nev, sorted
-// by output) mark where a column's output range starts (q + 1) or ends (-(q + 1)).
-void recombine_p(double* Xp, int64_t n, const double* Z, const double* Zp, const double* W,
-                 int64_t gstride, const RoundCols& rc, const int32_t* ev_o, const int32_t* ev_q,
-                 int nev, int o_begin, int o_end, double dt_out, cudaStream_t st);
-constexpr double kTcMinCover = 0.25;  // least share of a round's (column, output) pairs its
-                                      // columns cover for the dense tensor-core product to pay
+constexpr int kRmMaxSteps = 56;  // K steps (16 terms) of one launch
+constexpr int kRmMaxOutputs = 8192;  // outputs whose tables leave a launch room for 24 K steps at least
+struct RmScratch {
+  RmK* list = nullptr;                  // the round's terms
+  unsigned char* tiles = nullptr;       // coefficient tiles of one launch
+  int16_t* exps = nullptr;              // and their exponents
+  unsigned long long* mask = nullptr;   // K steps of every output tile, per launch
+};
+size_t rm_tiles_bytes(int n_times);
+size_t rm_exps(int n_times);
+bool rm_set_limits();
+// Xp[o][i] += the round's columns (V y and -P) at outputs [obeg_min, oend_max);
+// kdim = sum of mcol; order (or null): the columns by first output; pbound: the
+// columns' largest |z - w| and |z'| (krylov_start); tcut as recombine.  Returns the number of kernels launched.
+int recombine_mma(double* Xp, int64_t n, const double* Vbase, int64_t vstride, const double* Z,
+                  const double* Zp, const double* W, int64_t gstride, const RoundCols& rc,
+                  const int32_t* order, const int32_t* mcol, const double* coef, int ldo, int K,
+                  int kdim, int obeg_min, int oend_max, const RmScratch& rs, cudaStream_t st,
+                  const double* pbound, const int32_t* tcut);
+// Where the tensor cores take a round: from 4 terms per output on average (the
+// FP64 kernel's time is the terms, about 2.5 ms per 180k nodes, 1,000 outputs and
+// 4 terms; the tensor cores' a tile's conversion and X, whatever the terms up to
+// 16).  Five single-layer grids: 16.9 ms together at 4, 18.1 at 8, 19.1 at 12,
+// 23.4 at 16, 25.3 with the FP64 kernel alone.  Below 2e6 products the FP64
+// kernel takes less than the three launches.
+constexpr double kRmDensity = 4.0, kRmMinWork = 2e6;
+constexpr int kTcMinKdim = 16;         // a round counts as dense from this many basis vectors
+constexpr double kTcMinCover = 0.25;   // and this share of its (column, output) pairs held
 
 // Adjoint checkpoints: CK[q] = {X[groups[q]], Z[groups[q]]} ([K][2][n]), or the
 // reverse copy when restore is set (X, Z per group, [G][n]).

@@ -46,7 +46,7 @@ struct Round {
   int32_t K;      // columns
   int32_t obeg_min, oend_max;
   double cover = 0.0;          // share of (column, output) pairs of the range the columns hold
-  int32_t ev_begin = 0, nev = 0;  // -P events of the round (recombine_p)
+  double held = 0.0;           // those pairs
 };
 
 // Device address of the allocation-free solve's static scratch array on
@@ -102,8 +102,8 @@ struct matex_ctx {
   K1Plan k1;
   std::vector<int32_t> k1_fw_off, k1_bw_off;
   bool k1_use = false;
-  TcScratch tc;                    // tensor-core recombination (kdim_cap 0: not used)
-  int32_t *ev_o_d = nullptr, *ev_q_d = nullptr;  // -P events of all rounds
+  RmScratch rm;                    // tensor-core recombination (list null: not used)
+  int32_t* rc_order = nullptr;     // per round of `rounds`: its columns by first output
   // persistent solve: per column count (1..ldy) one PersistLevel row per level
   PersistLevel* plev_d = nullptr;
   std::vector<long long> pf_total, pb_total;   // per column count
@@ -1729,7 +1729,7 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
     // segment: z_j = z_{j-1} + L_{j-1} z'_{j-1}, z_0 = x(0)); then
     // z' = G^{-1} B s_j and w = G^{-1} C z'   (Eq. 5/6)
     e = prof_begin(c);
-    advance_z(c->Zb, c->Zpb, c->Xb, n, rc, K, n, st);
+    advance_z(c->Zb, c->Zpb, c->Xb, n, rc, K, n, c->pbound, st);
     if (c->opts.tape == 2 && !c->serial && ri % (size_t)c->tape_W == 0) {
       // adjoint checkpoint: x and z of every column at the start of the window
       checkpoint_states(c->CK + c->ck_base[ri / c->tape_W] * 2 * n, c->Xb, c->Zb, rc.group, K, n,
@@ -1752,7 +1752,7 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
     sweepsG += 2;
     // start vector v = x + F, beta = ||v||
     e = prof_begin(c);
-    krylov_start(c->Vb, vstride, c->Xb, c->Zb, c->Wb, n, rc.group, rc.vslot, K, n, c->partials,
+    krylov_start(c->Vb, vstride, c->Xb, c->Zb, c->Zpb, c->Wb, c->pbound, n, rc.group, rc.vslot, K, n, c->partials,
                  c->nchunks, st);
     prof_end(c, e, P_OTHER, 1, 4.0 * nd * K, 32.0 * nd * K);
     e = prof_begin(c);
@@ -1821,28 +1821,21 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
     if (c->opts.tape == 1) tape_small(c->ss, rc, K, c->THt, c->Tbeta, st);
     e = prof_begin(c);
     const double teps = c->opts.tail_eps;
-    if (teps > 0.0) {
-      e = prof_begin(c);
-      p_bound(c->Zb, c->Zpb, c->Wb, n, rc, K, n, c->pbound, st);
-      prof_end(c, e, P_OTHER, 1, 3.0 * nd * K, 24.0 * nd * K);
-      launches++;
-    }
     e = prof_begin(c);
     output_coefficients(c->ss, rc, K, c->gamma, c->dt_out, c->coef, c->n_times, c->yend, st,
                         teps, teps > 0.0 ? c->pbound : nullptr, c->tcut);
     prof_end(c, e, P_SMALL, 1, 0.0, 0.0);
     e = prof_begin(c);
     int rl = 1;
-    if (c->tc.kdim_cap && teps == 0.0 && kdim >= kTcMinKdim && kdim <= c->tc.kdim_cap &&
-        r.cover >= kTcMinCover) {
-      // V y on the tensor cores (a dense product over the round's output
-      // range, worth it when the columns hold most of that range), then the
-      // -P terms alone in one sweep over the outputs
-      rl += recombine_tc(c->Xp, n, c->Vb, vstride, rc, c->ss.m, c->coef, c->n_times, K, kdim,
-                         r.obeg_min, r.oend_max, c->tc, st);
-      pc.tc_rounds++;
-      recombine_p(c->Xp, n, c->Zb, c->Zpb, c->Wb, n, rc, c->ev_o_d + r.ev_begin,
-                  c->ev_q_d + r.ev_begin, r.nev, r.obeg_min, r.oend_max, c->dt_out, st);
+    // The tensor cores from kRmDensity terms per output of the round's range
+    // (basis vectors and -P, on average) and kRmMinWork products in all.
+    const double terms = r.held * (kdim + 2.0 * K) / K;
+    if (c->rm.list && kdim > 0 && terms >= kRmDensity * (r.oend_max - r.obeg_min) &&
+        nd * terms >= kRmMinWork) {
+      rl = recombine_mma(c->Xp, n, c->Vb, vstride, c->Zb, c->Zpb, c->Wb, n, rc,
+                         c->serial ? nullptr : c->rc_order + r.begin, c->ss.m, c->coef, c->n_times, K,
+                         kdim, r.obeg_min, r.oend_max, c->rm, st, c->pbound, teps > 0.0 ? c->tcut : nullptr);
+      if (teps == 0.0 && kdim >= kTcMinKdim && r.cover >= kTcMinCover) pc.tc_rounds++;
     } else {
       recombine(c->Xp, n, c->n_times, c->Vb, vstride, c->Zb, c->Zpb, c->Wb, n, rc, c->ss.m, c->coef,
                 c->n_times, K, r.obeg_min, r.oend_max, c->dt_out, st,
@@ -2128,7 +2121,7 @@ matex_status recompute_window(matex_ctx* c, int w, int r0, int r1, const std::ve
     RoundCols rc = round_cols(c, sub);
     rc.vslot = c->iota_d + (int64_t)i * Kb;
     const int b0 = sub.begin;
-    if (r != r0) advance_z(c->Zb, c->Zpb, c->Xb, n, rc, K, n, st);
+    if (r != r0) advance_z(c->Zb, c->Zpb, c->Xb, n, rc, K, n, c->pbound, st);
     build_input_rhs(c->Y, c->ldy, K, rc, c->src, n, st);
     solve_cols(c, c->fG, K);
     scatter_cols(c->Y, c->ldy, K, c->Zpb, n, rc.group, nullptr, n, st);
@@ -2136,7 +2129,7 @@ matex_status recompute_window(matex_ctx* c, int w, int r0, int r1, const std::ve
     gather_cols(c->Y, c->ldy, K, c->Zpb, n, rc.group, c->c_perm, nullptr, n, st);
     solve_cols(c, c->fG, K);
     scatter_cols(c->Y, c->ldy, K, c->Wb, n, rc.group, nullptr, n, st);
-    krylov_start(c->Vb, vstride, c->Xb, c->Zb, c->Wb, n, rc.group, rc.vslot, K, n, c->partials,
+    krylov_start(c->Vb, vstride, c->Xb, c->Zb, c->Zpb, c->Wb, c->pbound, n, rc.group, rc.vslot, K, n, c->partials,
                  c->nchunks, st);
     int32_t* iter = c->iterA;
     int32_t* iter_next = c->iterB;
@@ -2594,35 +2587,24 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   c->h_nout_all = h_nout;
   c->h_segid_all = h_segid;
   c->h_group_all = h_group;
-  std::vector<int32_t> ev_o_h, ev_q_h;
+  std::vector<int32_t> order_h(h_group.size(), 0);
   for (Round& rd : c->rounds) {
     std::vector<char> cov(c->n_times, 0);
     int cnt = 0;
     double held = 0.0;
-    std::vector<std::pair<int32_t, int32_t>> ev;
     for (int q = 0; q < rd.K; ++q) {
       const int ob = h_obeg[rd.begin + q], no = h_nout[rd.begin + q];
       held += no;
-      if (no > 0) {
-        ev.push_back({ob, q + 1});
-        ev.push_back({ob + no, -(q + 1)});
-      }
       for (int o = ob; o < ob + no; ++o)
         if (!cov[o]) { cov[o] = 1; cnt++; }
+      order_h[rd.begin + q] = q;
     }
     c->round_cover.push_back(cnt);
     const int span = rd.oend_max - rd.obeg_min;
+    rd.held = held;
     rd.cover = span > 0 ? held / ((double)rd.K * span) : 0.0;
-    std::stable_sort(ev.begin(), ev.end(),
-                     [](const std::pair<int32_t, int32_t>& a, const std::pair<int32_t, int32_t>& b) {
-                       return a.first < b.first;
-                     });
-    rd.ev_begin = (int32_t)ev_o_h.size();
-    rd.nev = (int32_t)ev.size();
-    for (const auto& x : ev) {
-      ev_o_h.push_back(x.first);
-      ev_q_h.push_back(x.second);
-    }
+    std::stable_sort(order_h.begin() + rd.begin, order_h.begin() + rd.begin + rd.K,
+                     [&](int32_t a, int32_t b) { return h_obeg[rd.begin + a] < h_obeg[rd.begin + b]; });
   }
   c->offd_rows = c->S.sup_rowptr[c->S.nsup] - c->S.n;
   // the same column records, one group at a time in time order
@@ -2637,6 +2619,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
         one.K = 1;
         one.obeg_min = h_nout[rec] > 0 ? h_obeg[rec] : c->n_times;
         one.oend_max = h_nout[rec] > 0 ? h_obeg[rec] + h_nout[rec] : 0;
+        one.held = h_nout[rec];
         c->serial_rounds.push_back(one);
         c->serial_cover.push_back(h_nout[rec]);
       }
@@ -2709,8 +2692,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   ok = ok && c->upload(c->init_groups_d, c->init_groups.data(), c->init_groups.size());
   ok = ok && c->upload(c->init_slots_d, init_slots.data(), init_slots.size());
   ok = ok && c->upload(c->rc_sgroup, h_sgroup.data(), h_sgroup.size());
-  ok = ok && c->upload(c->ev_o_d, ev_o_h.data(), ev_o_h.size()) &&
-       c->upload(c->ev_q_d, ev_q_h.data(), ev_q_h.size());
+  ok = ok && c->upload(c->rc_order, order_h.data(), order_h.size());
   std::vector<int32_t> h_vslot(h_group.size());
   for (size_t r = 0; r < h_group.size(); ++r) h_vslot[r] = o.tape == 1 ? (int32_t)r : h_group[r];
   ok = ok && c->upload(c->rc_vslot, h_vslot.data(), h_vslot.size());
@@ -2818,29 +2800,17 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
     return MATEX_ERR_OOM;
   }
   set_small_smem_limits();
-  if (o.recombine == 0 && o.tail_eps == 0.0) {
-    // tensor-core recombination scratch, sized once for rounds of up to
-    // kdim_cap basis vectors (never regrown: recorded graphs keep pointers)
-    int cap = std::min(Kmax * m_max, kTcMaxKdim);
-    cap = (cap + 31) & ~31;
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    while (cap > 32 && (double)tc_slices_bytes(n, cap, c->n_times) > 0.3 * (double)free_b) cap -= 32;
-    if (cap >= kTcMinKdim &&
-        (double)tc_slices_bytes(n, cap, c->n_times) <= 0.3 * (double)free_b) {
-      unsigned char* sl = nullptr;
-      int64_t* km = nullptr;
-      int32_t* kq = nullptr;
-      double *rsc = nullptr, *csc = nullptr;
-      const size_t ncol = ((size_t)c->n_times + 47) / 48 * 48;
-      if (c->alloc(sl, tc_slices_bytes(n, cap, c->n_times)) && c->alloc(km, cap) &&
-          c->alloc(kq, cap) && c->alloc(rsc, n) && c->alloc(csc, ncol)) {
-        c->tc = TcScratch{sl, km, kq, rsc, csc, c->d_count + 1, cap};
-        tc_set_limits();
-      } else {
-        cudaGetLastError();  // no room: the FP64 recombination serves every round
-      }
-    }
+  if (o.recombine == 0) {
+    // tensor-core recombination: a round's terms (at most m_max + 2 per column)
+    // and the coefficient tiles of one launch
+    const size_t terms = ((size_t)Kmax * (m_max + 2) + 15) / 16 * 16;
+    RmScratch rs;
+    if (c->n_times <= kRmMaxOutputs && rm_set_limits() && c->alloc(rs.list, terms) &&
+        c->alloc(rs.tiles, rm_tiles_bytes(c->n_times)) && c->alloc(rs.exps, rm_exps(c->n_times)) &&
+        c->alloc(rs.mask, (terms / 16 + 1) * ((c->n_times + 15) / 16)))
+      c->rm = rs;
+    else
+      cudaGetLastError();  // no room: the FP64 recombination serves every round
   }
   c->ss.krylov = o.krylov;
   c->ss.rscale = o.krylov == 1 ? 1.0 / gamma : o.krylov == 2 ? gamma : 1.0;
