@@ -103,65 +103,6 @@ krylov_start_kernel(double* __restrict__ Vb, int64_t vstride, const double* __re
   if (threadIdx.x == 0) partials[(int64_t)q * nchunks + blockIdx.x] = s;
 }
 
-// Dot products of w (slot wslot) with NB basis slots first..first+NB-1 over one
-// chunk of nodes; NB is a template parameter so no predicated FP64 work is
-// issued for slots that do not exist (the FP64 pipe counts those too).
-template <int NB>
-__device__ __forceinline__ void dots_chunk(const double* __restrict__ base, const double* __restrict__ w,
-                                           int first, int64_t n, int64_t b, int64_t e,
-                                           double* __restrict__ out, int nchunks, double* red) {
-  double acc[NB];
-#pragma unroll
-  for (int i = 0; i < NB; ++i) acc[i] = 0.0;
-  for (int64_t x = b + threadIdx.x; x < e; x += blockDim.x) {
-    const double wx = w[x];
-#pragma unroll
-    for (int i = 0; i < NB; ++i) acc[i] = fma(base[(int64_t)(first + i) * n + x], wx, acc[i]);
-  }
-#pragma unroll
-  for (int i = 0; i < NB; ++i) {
-    const double s = block_sum(acc[i], red);
-    if (threadIdx.x == 0) out[(int64_t)i * nchunks] = s;
-  }
-}
-
-__global__ void __launch_bounds__(kRedThreads)
-basis_dots_kernel(const double* __restrict__ Vb, int64_t vstride, const int32_t* __restrict__ groups,
-                  const int32_t* __restrict__ iter, int first, int nb, int wslot, int64_t n,
-                  double* __restrict__ partials, int nchunks) {
-  __shared__ double red[32];
-  const int q = iter[blockIdx.y];
-  const int64_t g = groups[q];
-  const double* __restrict__ base = Vb + g * vstride;
-  const double* __restrict__ w = base + (int64_t)wslot * n;
-  const int64_t b = (int64_t)blockIdx.x * kChunk;
-  const int64_t e = min(n, b + kChunk);
-  double* out = partials + ((int64_t)q * kMaxB) * nchunks + blockIdx.x;
-  switch (nb) {
-#define MATEX_DC(NB) \
-  case NB: dots_chunk<NB>(base, w, first, n, b, e, out, nchunks, red); break;
-    MATEX_DC(1) MATEX_DC(2) MATEX_DC(3) MATEX_DC(4) MATEX_DC(5) MATEX_DC(6) MATEX_DC(7)
-    MATEX_DC(8) MATEX_DC(9) MATEX_DC(10) MATEX_DC(11) MATEX_DC(12) MATEX_DC(13) MATEX_DC(14)
-    MATEX_DC(15) MATEX_DC(16) MATEX_DC(17) MATEX_DC(18) MATEX_DC(19) MATEX_DC(20) MATEX_DC(21)
-#undef MATEX_DC
-    default: break;
-  }
-}
-
-__global__ void basis_update_kernel(double* __restrict__ Vb, int64_t vstride,
-                                    const int32_t* __restrict__ groups,
-                                    const int32_t* __restrict__ iter, int nb, int wslot,
-                                    const double* __restrict__ h, int64_t n) {
-  const int q = iter[blockIdx.y];
-  const int64_t g = groups[q];
-  double* __restrict__ base = Vb + g * vstride;
-  const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= n) return;
-  double acc = base[(int64_t)wslot * n + x];
-  for (int i = 0; i < nb; ++i) acc = fma(-h[q * kMaxB + i], base[(int64_t)i * n + x], acc);
-  base[(int64_t)wslot * n + x] = acc;
-}
-
 __global__ void basis_scale_kernel(double* __restrict__ Vb, int64_t vstride,
                                    const int32_t* __restrict__ groups,
                                    const int32_t* __restrict__ iter, int wslot,
@@ -255,25 +196,6 @@ start_finish_kernel(const double* __restrict__ partials, int nchunks, int K, Sma
   if (last_cta(ca.arrived)) compact_columns(ss, ca, nullptr, K);
 }
 
-__global__ void reduce_dots_kernel(const double* __restrict__ partials, int nchunks, int nb,
-                                   const int32_t* __restrict__ iter, SmallState ss, int j,
-                                   int mode) {
-  const int q = iter[blockIdx.x];
-  const int i = threadIdx.x;
-  if (i >= nb) return;
-  double s = 0.0;
-  for (int k = 0; k < nchunks; ++k) s += partials[((int64_t)q * kMaxB + i) * nchunks + k];
-  double* Ht = ss.Ht + (int64_t)q * kMaxB * kMaxM;
-  if (mode == 2) {
-    const double nrm = sqrt(s);
-    Ht[(j + 1) * kMaxM + j] = nrm;
-    ss.scale[q] = nrm > 0.0 ? 1.0 / nrm : 0.0;
-  } else {
-    ss.hbuf[q * kMaxB + i] = s;
-    Ht[i * kMaxM + j] += s;
-  }
-}
-
 __global__ void __launch_bounds__(kTeamThreads)
 residual_kernel(SmallState ss, RoundCols rc, const int32_t* __restrict__ iter, int j, double gamma,
                 double tol, int m_max, const int32_t* __restrict__ replay, CompactArgs ca) {
@@ -344,20 +266,6 @@ void krylov_start(double* Vbase, int64_t vstride, const double* X, const double*
       vslots, n, partials, nchunks);
 }
 
-void basis_dots(const double* Vbase, int64_t vstride, const int32_t* groups, const int32_t* iter,
-                int K, int first, int nb, int wslot, int64_t n, double* partials, int nchunks,
-                cudaStream_t st) {
-  dim3 grid((unsigned)nchunks, (unsigned)K);
-  basis_dots_kernel<<<grid, kRedThreads, 0, st>>>(Vbase, vstride, groups, iter, first, nb, wslot,
-                                                  n, partials, nchunks);
-}
-
-void basis_update(double* Vbase, int64_t vstride, const int32_t* groups, const int32_t* iter, int K,
-                  int nb, int wslot, const double* h, int64_t n, cudaStream_t st) {
-  dim3 grid((unsigned)((n + 255) / 256), (unsigned)K);
-  basis_update_kernel<<<grid, 256, 0, st>>>(Vbase, vstride, groups, iter, nb, wslot, h, n);
-}
-
 void basis_scale(double* Vbase, int64_t vstride, const int32_t* groups, const int32_t* iter, int K,
                  int wslot, const double* scale, int64_t n, cudaStream_t st) {
   dim3 grid((unsigned)((n + 255) / 256), (unsigned)K);
@@ -367,11 +275,6 @@ void basis_scale(double* Vbase, int64_t vstride, const int32_t* groups, const in
 void start_finish(const double* partials, int nchunks, int K, SmallState ss, const CompactArgs& ca,
                   cudaStream_t st) {
   start_finish_kernel<<<K, kRedThreads, 0, st>>>(partials, nchunks, K, ss, ca);
-}
-
-void reduce_dots(const double* partials, int nchunks, int K, int nb, const int32_t* iter,
-                 SmallState ss, int j, int mode, cudaStream_t st) {
-  reduce_dots_kernel<<<K, 32, 0, st>>>(partials, nchunks, nb, iter, ss, j, mode);
 }
 
 namespace {

@@ -194,14 +194,6 @@ void krylov_start(double* Vbase, int64_t vstride, const double* X, const double*
                   const double* W, double* pbound, int64_t gstride, const int32_t* groups, const int32_t* vslots,
                   int K, int64_t n, double* partials, int nchunks, cudaStream_t st);
 
-// Partial dot products of basis slot wslot (w) with slots first..first+nb-1
-// for each iterating column; partials laid out [K][kMaxB][nchunks].
-void basis_dots(const double* Vbase, int64_t vstride, const int32_t* groups, const int32_t* iter,
-                int K, int first, int nb, int wslot, int64_t n, double* partials, int nchunks,
-                cudaStream_t st);
-// w -= sum_i h[q][i] v_i  (h from coef, [K][kMaxB])
-void basis_update(double* Vbase, int64_t vstride, const int32_t* groups, const int32_t* iter,
-                  int K, int nb, int wslot, const double* h, int64_t n, cudaStream_t st);
 // V[wslot] *= scale[q]
 void basis_scale(double* Vbase, int64_t vstride, const int32_t* groups, const int32_t* iter,
                  int K, int wslot, const double* scale, int64_t n, cudaStream_t st);
@@ -214,7 +206,6 @@ struct SmallState {
   double* beta;      // [ncol]
   int32_t* m;        // [ncol] current / final Krylov dimension (0 = quiescent)
   int32_t* status;   // [ncol] 0 iterating, 1 converged, 2 breakdown, 3 m_max, 4 quiescent
-  double* hbuf;      // [ncol][kMaxB] Gram-Schmidt coefficients of the current pass
   double* scale;     // [ncol] 1/norm for normalisation
   int32_t krylov = 0;   // Krylov space: 0 rational, 1 inverted, 2 standard (exponent map)
   double rscale = 1.0;  // factor on h_{m+1,m} in the residual: 1, 1/gamma, gamma
@@ -237,9 +228,13 @@ struct CompactArgs {
 // lists the non-quiescent columns
 void start_finish(const double* partials, int nchunks, int K, SmallState ss, const CompactArgs& ca,
                   cudaStream_t st);
-// reduce dot partials into hbuf (and accumulate into Ht column j when acc != 0)
-void reduce_dots(const double* partials, int nchunks, int K, int nb, const int32_t* iter,
-                 SmallState ss, int j, int mode, cudaStream_t st);
+// Orthogonalise slot nb of each iterating column against its slots 0..nb-1 (two
+// classical Gram-Schmidt passes), then normalise it; column nb - 1 of Ht gets
+// the coefficients and the norm (a zero or NaN norm scales by 0).  partials: the
+// doubles of gram_schmidt_partials for at least K columns.  Returns the launches.
+size_t gram_schmidt_partials(int K, int64_t n);
+int gram_schmidt(double* Vb, int64_t vstride, const int32_t* slots, const int32_t* iter, int K,
+                 int nb, int64_t n, SmallState ss, double* partials, cudaStream_t st);
 // w = A v = -C^{-1} G v for the standard Krylov space: column q of the batch
 // reads slot `jsrc` of its basis and writes slot `jdst` (G in CSR, permuted).
 void krylov_apply_A(double* Vb, int64_t vstride, const int32_t* iter_grp, int K, int jsrc, int jdst,

@@ -1799,22 +1799,13 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
       sweepsM++;
       // two classical Gram-Schmidt passes, then the norm and the normalisation
       e = prof_begin(c);
-      for (int pass = 0; pass < 2; ++pass) {
-        basis_dots(c->Vb, vstride, rc.vslot, iter, kit, 0, j + 1, j + 1, n, c->partials,
-                   c->nchunks, st);
-        reduce_dots(c->partials, c->nchunks, kit, j + 1, iter, c->ss, j, pass, st);
-        basis_update(c->Vb, vstride, rc.vslot, iter, kit, j + 1, j + 1, c->ss.hbuf, n, st);
-      }
-      basis_dots(c->Vb, vstride, rc.vslot, iter, kit, j + 1, 1, j + 1, n, c->partials, c->nchunks,
-                 st);
-      reduce_dots(c->partials, c->nchunks, kit, 1, iter, c->ss, j, 2, st);
-      basis_scale(c->Vb, vstride, rc.vslot, iter, kit, j + 1, c->ss.scale, n, st);
-      prof_end(c, e, P_GS, 9, (8.0 * j + 11.0) * nd * kit, (4.0 * j + 13.0) * 8.0 * nd * kit);
+      const int gl = gram_schmidt(c->Vb, vstride, rc.vslot, iter, kit, j + 1, n, c->ss, c->partials, st);
+      prof_end(c, e, P_GS, gl, (8.0 * j + 11.0) * nd * kit, (3.0 * j + 10.0) * 8.0 * nd * kit);
       e = prof_begin(c);
       residual_check(c->ss, rc, kit, j, c->gamma, c->tol, c->m_max, c->replay_d, iter,
                      next_list(iter_next, rc.vslot), st);
       prof_end(c, e, P_SMALL, 1, 0.0, 0.0);
-      launches += 10;
+      launches += gl + 2;
       std::swap(iter, iter_next);
       if ((s = count(&kit)) != MATEX_OK) return s;
     }
@@ -2152,16 +2143,7 @@ matex_status recompute_window(matex_ctx* c, int w, int r0, int r1, const std::ve
                    n, st);
       scatter_cols(c->Y, c->ldy, kit, c->TA + (int64_t)j * n, (int64_t)kMaxM * n, c->iter_grp,
                    nullptr, n, st);
-      for (int pass = 0; pass < 2; ++pass) {
-        basis_dots(c->Vb, vstride, rc.vslot, iter, kit, 0, j + 1, j + 1, n, c->partials,
-                   c->nchunks, st);
-        reduce_dots(c->partials, c->nchunks, kit, j + 1, iter, c->ss, j, pass, st);
-        basis_update(c->Vb, vstride, rc.vslot, iter, kit, j + 1, j + 1, c->ss.hbuf, n, st);
-      }
-      basis_dots(c->Vb, vstride, rc.vslot, iter, kit, j + 1, 1, j + 1, n, c->partials, c->nchunks,
-                 st);
-      reduce_dots(c->partials, c->nchunks, kit, 1, iter, c->ss, j, 2, st);
-      basis_scale(c->Vb, vstride, rc.vslot, iter, kit, j + 1, c->ss.scale, n, st);
+      gram_schmidt(c->Vb, vstride, rc.vslot, iter, kit, j + 1, n, c->ss, c->partials, st);
       const int left = active(j + 1);
       residual_check(c->ss, rc, kit, j, c->gamma, c->tol, c->m_max, c->m_rec, iter,
                      next_list(iter_next, left), st);
@@ -2733,7 +2715,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
     const double nd = (double)n;
     const double run_b = 8.0 * (2.0 * nd * c->ldy + (double)G * kMaxB * nd + 4.0 * G * nd +
                                 (double)c->n_times * nd + (double)Kmax * c->n_times * kCoefLd +
-                                (double)Kmax * kMaxB * c->nchunks);
+                                (double)gram_schmidt_partials(Kmax, n));
     const double budget = 0.85 * ((double)free_b - run_b);
     const TapePlan tp = plan_tape(c->rounds, n, (int)G, Kmax, c->n_times, c->nrows_out, budget,
                                   o.tape_window, o.tape_block);
@@ -2758,10 +2740,10 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   ok = ok && c->alloc(c->Y, (size_t)n * c->ldy) && c->alloc(c->Y2, (size_t)n * c->ldy) && c->alloc(c->Vb, vslots * kMaxB * n) &&
        c->alloc(c->Zb, G * n) && c->alloc(c->Zpb, G * n) && c->alloc(c->Wb, G * n) &&
        c->alloc(c->Xb, G * n) && c->alloc(c->Xp, (size_t)c->n_times * n) && c->alloc(c->xdc, n) &&
-       c->alloc(c->partials, (size_t)Kmax * kMaxB * c->nchunks) &&
+       c->alloc(c->partials, std::max((size_t)Kmax * kMaxB * c->nchunks, gram_schmidt_partials(Kmax, n))) &&
        c->alloc(c->ss.Ht, (size_t)Kmax * kMaxB * kMaxM) && c->alloc(c->ss.beta, Kmax) &&
        c->alloc(c->ss.m, Kmax) && c->alloc(c->ss.status, Kmax) &&
-       c->alloc(c->ss.hbuf, (size_t)Kmax * kMaxB) && c->alloc(c->ss.scale, Kmax) &&
+       c->alloc(c->ss.scale, Kmax) &&
        c->alloc(c->iterA, Kmax) && c->alloc(c->iterB, Kmax) && c->alloc(c->iter_grp, Kmax) &&
        c->alloc(c->d_count, 4) && c->alloc(c->coef, (size_t)Kmax * c->n_times * kCoefLd) &&
        c->alloc(c->yend, (size_t)Kmax * kMaxM) &&
