@@ -545,7 +545,7 @@ struct MmSup {
 };
 constexpr int kMmCols = 16;         // right-hand sides of a thread block
 constexpr int kMmPack = 8;          // supernodes of a packed task (their K steps fit one chunk)
-constexpr int kMmRowsWide = 32, kMmRowsNarrow = 4;  // most row tiles of a task, two versions
+constexpr int kMmRowsWide = 24, kMmRowsNarrow = 4;  // most row tiles of a task, two versions
 // Flag in a node index: backward, read x of an ancestor from Y (without it
 // y_s from Y2); forward, subtract from an ancestor's row of Y.
 constexpr int kMmAdd = 1 << 30;
@@ -565,11 +565,30 @@ struct MmLevel {
   int32_t nmulti = 0, nsingle = 0, steps = 1;
 };
 // A level takes its wide tasks from 3 CTAs per SM on (below, narrow ones spread
-// the level further; 6 and 12 a SM measured 2 and 8 % slower at 64 columns on
-// the 180k-node grid), a cluster shares a task's K steps while that adds CTAs
-// up to 2 per SM (1: 5 % slower, 4: 4 %), at least two steps each, and the
-// ring of panel tiles is deep up to 3 CTAs per SM, all of them resident at once.
-constexpr int kMmFill = 3 * 152, kMmClusterFill = 2 * 152, kMmDeep = 3 * 152;
+// the level further; from 2 on 5 % slower at 64 columns on the 180k-node grid,
+// from 5 on with 16 row tiles no faster), a cluster shares a task's K steps while
+// that adds CTAs up to 3 per SM (2: 2 % slower at 16 and 64 columns), at least
+// two steps each, and levels of narrow tasks up to 2 CTAs per SM, all of them
+// resident at once, take the eight-warp kernel (up to 3, so in two waves: 5 %
+// slower at 8 columns on 40,000 nodes).
+constexpr int kMmFill = 3 * 152, kMmClusterFill = 3 * 152, kMmDeep = 2 * 152;
+// The K steps [ka, kz) of a task of K steps [kbeg, kend) that CTA `rank` of a
+// cluster of cs takes: steps rank p .. rank p + p - 1 from the multiple of p at
+// or below kbeg, p the smallest power of two with which cs CTAs reach kend, or a
+// number of whole chunks (8 steps).  A piece then never crosses a chunk's end
+// unless it holds whole chunks: two pieces cost the splitting of their
+// right-hand sides twice (2,600 clocks, as long as six K steps).
+__host__ __device__ inline void mm_share(int kbeg, int kend, int rank, int cs, int& ka, int& kz) {
+  constexpr int kCh = 8;
+  int p = 1;
+  while (p < kCh && (kbeg & -p) + cs * p < kend) p *= 2;
+  const int base = kbeg & -p;
+  if (p == kCh) p = kCh * ((kend - base + kCh * cs - 1) / (kCh * cs));
+  ka = base + rank * p;
+  kz = ka + p;
+  ka = ka < kbeg ? kbeg : ka > kend ? kend : ka;
+  kz = kz > kend ? kend : kz;
+}
 struct MmPlan {
   int32_t nlev = 0, nsup = 0;
   const MmSup* sups[2] = {};             // per direction (0 forward), in task order

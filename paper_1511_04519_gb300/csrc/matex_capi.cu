@@ -3403,8 +3403,8 @@ extern "C" matex_status matex_host_tensor_plan(int64_t n, const int64_t* rowptr,
         part.assign((size_t)tk.nu * 8 * ncols, 0.0);
         const int cs = multi ? cluster : 1;
         for (int rank = 0; rank < cs; ++rank) {
-          const int ka = tk.kbeg + (tk.kend - tk.kbeg) * rank / cs;
-          const int kz = tk.kbeg + (tk.kend - tk.kbeg) * (rank + 1) / cs;
+          int ka, kz;
+          mm_share(tk.kbeg, tk.kend, rank, cs, ka, kz);
           const int chb = ka / kCh, che = ka < kz ? (kz - 1) / kCh + 1 : chb;
           if (!multi && che - chb != 1) ++errors;
           for (int ch = chb; ch < che; ++ch) {

@@ -94,7 +94,7 @@ __device__ __forceinline__ void mma(float (&c)[4][kDigits], int d, const uint4& 
       : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-// rare results: zero, subnormal, overflow, a column that held an inf or NaN
+// rare results: subnormal, overflow, a column that held an inf or NaN
 static __device__ __noinline__ double compose_slow(long long s, int e) {
   if (e >= kNonFinite / 2) return __longlong_as_double(0x7ff8000000000000ll);
   return s == 0 ? 0.0 : ldexp((double)s, e - 2096);
@@ -116,10 +116,12 @@ __device__ __forceinline__ double compose(const float (&c)[kDigits], int e) {
   s += (long long)v[3] * 65536;
   s += (long long)(v[1] * 256 + v[2]) * 16777216;
   s += (long long)v[0] << 40;
-  // exponent fields of (double)s: 1023 .. 1085
-  if (s == 0 || (unsigned)(e - 1074) > 1982u) return compose_slow(s, e);
+  // exponent fields of (double)s: 1023 .. 1085; zeros (padded rows, unloaded
+  // nodes) are common and stay out of the call
+  const bool zero = s == 0 && e < kNonFinite / 2;
+  if (!zero && (unsigned)(e - 1074) > 1982u) return compose_slow(s, e);
   const double x = (double)s;
-  return __hiloint2double(__double2hiint(x) + (e - 2096) * (1 << 20), __double2loint(x));
+  return zero ? 0.0 : __hiloint2double(__double2hiint(x) + (e - 2096) * (1 << 20), __double2loint(x));
 }
 
 }  // namespace s8

@@ -82,3 +82,15 @@ def test_scales_zeros_and_non_finite_columns(M):
     assert not np.isfinite(x[4]).all() and not np.isfinite(x[5]).all()
     good = [0, 1, 2, 3, 6, 7, 8]
     assert np.isfinite(x[good]).all() and not x[2].any()
+
+
+@pytest.mark.parametrize("ncols", [1, 8, 9, 40, 130])
+def test_wide_separators(M, ncols):
+    # a 512-column top and reductions of up to 32 K steps: clusters of 2 to 8 with
+    # pieces of one chunk or several, the eight- and the four-warp kernel
+    p = _grid(4, 50, 48)
+    on = M.Sim(p, tc_solve="on", resident="off")
+    off = M.Sim(p, tc_solve="off", resident="off")
+    rng = np.random.default_rng(ncols)
+    for which in (0, 1):
+        _check(M, p, on, off, which, rng.standard_normal((ncols, p.n)))
