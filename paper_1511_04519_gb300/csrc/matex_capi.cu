@@ -1214,13 +1214,18 @@ RoundCols round_cols(matex_ctx* c, const Round& r) {
   return rc;
 }
 
+// the error flag among the counters that were copied last
+matex_status check_flags(matex_ctx* c) {
+  if (c->h_count[1] != 0)
+    return fail(c, MATEX_ERR_TIMEOUT, "a bounded wait of the persistent solve expired");
+  return MATEX_OK;
+}
+
 matex_status read_count(matex_ctx* c, int* out) {
   cudaMemcpyAsync(c->h_count, c->d_count, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->st);
   if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check(c, "sync");
   *out = c->h_count[0];
-  if (c->h_count[1] != 0)
-    return fail(c, MATEX_ERR_TIMEOUT, "a bounded wait of the persistent solve expired");
-  return MATEX_OK;
+  return check_flags(c);
 }
 
 // Algorithmic work of one batched solve pair with K right-hand sides, from
@@ -3025,11 +3030,13 @@ matex_status matex_solve(matex_ctx* c, int32_t which, int32_t ncols, const doubl
     solve_cols(c, F, K);
     scatter_cols(c->Y, c->ldy, K, x + (int64_t)q0 * n, n, nullptr, c->perm, n, c->st);
   }
+  // the flags follow the solution, for one synchronisation (a second copy and
+  // wait after it took 10 us of a call)
+  cudaMemcpyAsync(c->h_count, c->d_count, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->st);
   if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check(c, "solve sync");
   matex_status s = cuda_check(c, "solve");
   if (s != MATEX_OK) return s;
-  int tmp = 0;
-  return read_count(c, &tmp);
+  return check_flags(c);
 }
 
 matex_status matex_solve_resident(matex_ctx* c, int32_t which, int32_t ncols, const double* b,
