@@ -86,6 +86,7 @@ struct matex_ctx {
   // level solves on the tensor cores (opts.tc_solve, k_sptrsv_mma.cu): plan,
   // panel digits, and per column count whether a solve takes them
   MmPlan mm;
+  double* mm_pan = nullptr;  // a factor's panels on their way into digits
   bool mm_ok = false;
   std::vector<int8_t> mm_by_ncols;
   ResidentPlan rplan;
@@ -1044,17 +1045,10 @@ void build_mm_plan(const Symbolic& S, bool fwd, MmHostPlan& P) {
 
 // Both directions' panel tiles of factor fi from its coarse panels (host).
 bool load_mm(matex_ctx* c, int fi, const std::vector<double>& pan) {
-  double* p = nullptr;
-  if (cudaMalloc(&p, sizeof(double) * std::max<size_t>(1, pan.size())) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  bool ok = cudaMemcpy(p, pan.data(), sizeof(double) * pan.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+  bool ok = cudaMemcpy(c->mm_pan, pan.data(), sizeof(double) * pan.size(), cudaMemcpyHostToDevice) == cudaSuccess;
   for (int dir = 0; ok && dir < 2; ++dir)
-    mm_split_panels(p, (fi == 0 ? c->fM : c->fG).dinv, c->mm, dir == 0, c->mm.A[fi][dir], c->st);
-  ok = cudaStreamSynchronize(c->st) == cudaSuccess && ok;
-  cudaFree(p);
-  return ok;
+    mm_split_panels(c->mm_pan, (fi == 0 ? c->fM : c->fG).dinv, c->mm, dir == 0, c->mm.A[fi][dir], c->st);
+  return cudaStreamSynchronize(c->st) == cudaSuccess && ok;
 }
 
 // The plan and both factors' tiles.  False when there is no room (at most a
@@ -1066,7 +1060,8 @@ bool plan_mm(matex_ctx* c, const std::vector<double>& panM, const std::vector<do
     build_mm_plan(S, dir == 0, H[dir]);
     if (H[dir].tiles > INT32_MAX) return false;
   }
-  const double need = 2.0 * (double)mm_tile_bytes() * (double)(H[0].tiles + H[1].tiles);
+  const double need = 2.0 * (double)mm_tile_bytes() * (double)(H[0].tiles + H[1].tiles) +
+                      8.0 * (double)panM.size();
   size_t free_b = 0, total_b = 0;
   cudaMemGetInfo(&free_b, &total_b);
   if (need > 0.25 * (double)free_b || !mm_set_limits()) return false;
@@ -1093,6 +1088,8 @@ bool plan_mm(matex_ctx* c, const std::vector<double>& panM, const std::vector<do
     for (int fi = 0; fi < 2; ++fi)
       if (!c->alloc(c->mm.A[fi][dir], (size_t)H[dir].tiles * mm_tile_bytes())) return false;
   }
+  // kept for new capacitances, which then cannot fail for lack of memory
+  if (!c->alloc(c->mm_pan, std::max(panM.size(), panG.size()))) return false;
   return load_mm(c, 0, panM) && load_mm(c, 1, panG);
 }
 
