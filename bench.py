@@ -210,7 +210,7 @@ def measured_traffic():
     try:
         text = open(path).read()
         h = hashlib.sha256()
-        for f in ("k_sptrsv.cu", "k_sptrsv_k1.cu"):
+        for f in ("k_sptrsv.cu", "k_sptrsv_k1.cu", "k_sptrsv_mma.cu"):
             h.update(open(os.path.join(csrc, f), "rb").read())
         sha = h.hexdigest()[:16]
     except OSError as exc:
@@ -306,8 +306,7 @@ def ncu_case(what: str) -> int:
     kernel; "levels": 64 columns with one launch per tree level; "run": one
     full matex_run; "ksweep": bare solve pairs of 1, 4 and 64 columns on the
     whole grid; "small": one run of the 1,024-node single-group grid;
-    "tcsolve": one 64-column solve pair of the whole grid with the wide panels
-    on the tensor cores."""
+    "tcsolve": one 64-column solve pair of the whole grid on the tensor cores."""
     import numpy as np
     import torch
 
@@ -322,7 +321,7 @@ def ncu_case(what: str) -> int:
     q = gridgen.with_sources(p, p.src_node[sel], off, p.pwl_t.reshape(-1, 3)[sel].ravel(),
                              p.pwl_v.reshape(-1, 3)[sel].ravel(), p.src_group[sel], groups)
     if what == "tcsolve":
-        # the whole bench grid, wide panels forced onto the tensor cores: one
+        # the whole bench grid, every column count on the tensor cores: one
         # 64-column solve pair of C + gamma G after a warm one
         sim = M.Sim(p, tc_solve="on", solve_mode=1, include_dc=False,
                     rows=np.arange(4, dtype=np.int32))

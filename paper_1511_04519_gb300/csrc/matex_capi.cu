@@ -1096,9 +1096,9 @@ bool plan_mm(matex_ctx* c, const std::vector<double>& panM, const std::vector<do
 // Which solves take the tensor-core kernels.  opts.tc_solve 2: all (one column
 // only when opts.single_column does not force its own kernels); 0: from two
 // columns on, where they measured faster on every grid tried (1,024 to 180k
-// nodes: 1.2 to 1.6 times at two columns, 3.3 times at 16 and 64), and for one
+// nodes: 1.4 times and more at two columns, 3.5 times at 16 and 64), and for one
 // column where the pair is at least 5 % faster than the path chosen so far
-// (small grids: 0.049 against 0.062 ms on 1,024 nodes; 0.42 against 0.31 ms on
+// (small grids: 0.034 against 0.061 ms on 1,024 nodes; 0.37 against 0.31 ms on
 // 180k), cached in MATEX_AUTOTUNE_CACHE like the other choices.
 void choose_mm(matex_ctx* c) {
   c->mm_by_ncols.assign(c->ldy + 1, c->mm_ok ? 1 : 0);
