@@ -661,6 +661,12 @@ def main():
         1, d["units"])
     roof["algorithmic_bytes_per_launch"] = d["bytes"] / max(1, d["units"])
     traffic, traffic_src = measured_traffic() if dom == "solve" else (None, "not the solve class")
+    if dom == "solve" and roof["bound"] == "alu" and sim.setup_stats()["tc_solve_min_cols"]:
+        # above 1 of the FP64 pipe is possible: that pipe no longer does the products
+        roof["split_products_tflops"] = 34 * roof["achieved"]
+        roof["note"] = ("solves of two and more columns run as 34 FP16 products per FP64 product on "
+                        "the tensor cores (mma.sync, 600 TFLOP/s measured); the FP64 peak is the "
+                        "bound of the kernels they replace")
     roof["traffic"] = traffic
     roof["traffic_source"] = traffic_src
     s = prof["solve"]
