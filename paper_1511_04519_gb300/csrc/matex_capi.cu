@@ -261,12 +261,18 @@ struct matex_ctx {
     p = static_cast<T*>(q);
     return true;
   }
+  // Host to device on the context's stream, complete on return.  cudaMemcpy
+  // works on the legacy default stream, which a non-blocking stream does not
+  // wait for, and may return before the end of pageable memory has arrived.
+  template <typename T>
+  bool put(T* p, const T* h, size_t count) {
+    return count == 0 ||
+           (cudaMemcpyAsync(p, h, count * sizeof(T), cudaMemcpyHostToDevice, st) == cudaSuccess &&
+            cudaStreamSynchronize(st) == cudaSuccess);
+  }
   template <typename T>
   bool upload(T*& p, const T* h, size_t count) {
-    if (!alloc(p, count)) return false;
-    if (count && cudaMemcpy(p, h, count * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess)
-      return false;
-    return true;
+    return alloc(p, count) && put(p, h, count);
   }
 };
 
@@ -603,7 +609,7 @@ bool plan_levels(matex_ctx* c) {
   if (!c->upload(c->plev_d, pl.data(), pl.size())) return false;
   if (!c->alloc(c->split.part, (size_t)2 * kSplitSlots * kRowBlock * kMaxColBlock) ||
       !c->alloc(c->split.cnt, (size_t)kSplitSlots) ||
-      cudaMemset(c->split.cnt, 0, sizeof(int) * kSplitSlots) != cudaSuccess)
+      cudaMemsetAsync(c->split.cnt, 0, sizeof(int) * kSplitSlots, c->st) != cudaSuccess)
     return false;
   std::vector<int32_t> lev(S.nsup), nft(S.nsup), nbt(S.nsup), kids(S.nsup, 0);
   for (int l = 0; l < nlev; ++l)
@@ -1045,7 +1051,7 @@ void build_mm_plan(const Symbolic& S, bool fwd, MmHostPlan& P) {
 
 // Both directions' panel tiles of factor fi from its coarse panels (host).
 bool load_mm(matex_ctx* c, int fi, const std::vector<double>& pan) {
-  bool ok = cudaMemcpy(c->mm_pan, pan.data(), sizeof(double) * pan.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+  bool ok = c->put(c->mm_pan, pan.data(), pan.size());
   for (int dir = 0; ok && dir < 2; ++dir)
     mm_split_panels(c->mm_pan, (fi == 0 ? c->fM : c->fG).dinv, c->mm, dir == 0, c->mm.A[fi][dir], c->st);
   return cudaStreamSynchronize(c->st) == cudaSuccess && ok;
@@ -2752,7 +2758,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
        c->alloc(c->tcut, (size_t)Kmax * 2) && c->alloc(c->pbound, (size_t)Kmax * 2) && c->alloc(c->m_rec, std::max<int64_t>(1, c->n_segments)) &&
        c->alloc(c->st_rec, std::max<int64_t>(1, c->n_segments));
   if (ok && cudaMallocHost(&c->h_count, 4 * sizeof(int32_t)) != cudaSuccess) ok = false;
-  if (ok && cudaMemset(c->d_count, 0, 4 * sizeof(int32_t)) != cudaSuccess) ok = false;
+  if (ok && cudaMemsetAsync(c->d_count, 0, 4 * sizeof(int32_t), c->st) != cudaSuccess) ok = false;
   if (ok) c->fM.abort = c->fG.abort = c->d_count + 2;
   if (ok && o.tape) {
     // tape 1: one entry per record, reverse launches as wide as a round;
@@ -2881,8 +2887,8 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
     if (noalloc_scratch(c->device, &scratch, serr) != MATEX_OK) cudaGetLastError();
     preload_solve_kernels();
   }
-  cudaMemset(c->Vb, 0, sizeof(double) * vslots * kMaxB * n);
-  cudaMemset(c->Xb, 0, sizeof(double) * G * n);
+  cudaMemsetAsync(c->Vb, 0, sizeof(double) * vslots * kMaxB * n, c->st);
+  cudaMemsetAsync(c->Xb, 0, sizeof(double) * G * n, c->st);
   if (cudaDeviceSynchronize() != cudaSuccess) {
     g_setup_err = std::string("setup: ") + cudaGetErrorString(cudaGetLastError());
     delete c;
@@ -2916,15 +2922,11 @@ matex_status matex_set_caps(matex_ctx* c, const double* cap) {
   if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check(c, "set_caps sync");
   std::vector<double> cp(c->n);
   for (int64_t k = 0; k < c->n; ++k) cp[k] = cap[c->S.perm[k]];
-  bool ok = cudaMemcpy(const_cast<double*>(c->fM.dinv), NM.dinv.data(), sizeof(double) * NM.dinv.size(),
-                       cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(const_cast<double*>(c->fM.pan_cm), NM.pan_cm.data(),
-                       sizeof(double) * NM.pan_cm.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(const_cast<double*>(c->fM.pan_rm), NM.pan_rm.data(),
-                       sizeof(double) * NM.pan_rm.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(c->c_perm, cp.data(), sizeof(double) * c->n, cudaMemcpyHostToDevice) ==
-                cudaSuccess;
-  if (!ok) return cuda_check(c, "set_caps upload");
+  if (!c->put(const_cast<double*>(c->fM.dinv), NM.dinv.data(), NM.dinv.size()) ||
+      !c->put(const_cast<double*>(c->fM.pan_cm), NM.pan_cm.data(), NM.pan_cm.size()) ||
+      !c->put(const_cast<double*>(c->fM.pan_rm), NM.pan_rm.data(), NM.pan_rm.size()) ||
+      !c->put(c->c_perm, cp.data(), (size_t)c->n))
+    return cuda_check(c, "set_caps upload");
   if (c->mm_ok && !load_mm(c, 0, mm_pan)) return cuda_check(c, "set_caps tiles");
   if (c->resident_ok) {
     // the resident copy of the refactored C + gamma G
@@ -3659,12 +3661,9 @@ matex_status tr_prepare(matex_ctx* c, double h) {
     c->fT.abort = nullptr;
   }
   if (cudaStreamSynchronize(c->st) != cudaSuccess ||
-      cudaMemcpy(const_cast<double*>(c->fT.dinv), NT.dinv.data(), sizeof(double) * NT.dinv.size(),
-                 cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(const_cast<double*>(c->fT.pan_cm), NT.pan_cm.data(), sizeof(double) * NT.pan_cm.size(),
-                 cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(const_cast<double*>(c->fT.pan_rm), NT.pan_rm.data(), sizeof(double) * NT.pan_rm.size(),
-                 cudaMemcpyHostToDevice) != cudaSuccess)
+      !c->put(const_cast<double*>(c->fT.dinv), NT.dinv.data(), NT.dinv.size()) ||
+      !c->put(const_cast<double*>(c->fT.pan_cm), NT.pan_cm.data(), NT.pan_cm.size()) ||
+      !c->put(const_cast<double*>(c->fT.pan_rm), NT.pan_rm.data(), NT.pan_rm.size()))
     return cuda_check(c, "trapezoidal factor upload");
   c->tr_h = h;
   c->tr_factor_ms = now_ms() - t0;
