@@ -171,11 +171,29 @@ struct RmArgs {
   const unsigned char* tiles;
   const int16_t* exps;
   const unsigned long long* mask;
-  int ksteps, obeg, oend;
+  const double* coef;
+  int ldo, ksteps, obeg, oend;
   const int32_t* abort;
 };
 
-__global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const RmArgs a) {
+// Chunk ch of output o at node i in FP64, the terms that hold o alone: taken
+// where one of the chunk's values at i or of its coefficients at o is an inf or
+// NaN, which has no digits and may belong to a column that does not hold o.
+static __device__ __noinline__ double rm_plain(const RmArgs* a, int ch, int o, int64_t i) {
+  const int k1 = min(a->ksteps, (ch + 1) * kChunkSteps) * 16;
+  double s = 0.0;
+  for (int k = ch * kChunkSteps * 16; k < k1; ++k) {
+    const RmK e = a->list[k];
+    if (e.off < 0 || o < e.ob || o >= e.oe) continue;
+    const double v = e.j < kMaxM    ? a->Vb[e.off + i]
+                     : e.j == kMaxM ? a->Zp[e.off + i]
+                                    : a->Z[e.off + i] - a->W[e.off + i];
+    s = fma(v, e.j > kMaxM ? 1.0 : a->coef[((int64_t)e.q * a->ldo + (o - e.ob)) * kCoefLd + e.j], s);
+  }
+  return s;
+}
+
+__global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const __grid_constant__ RmArgs a) {
   // [K step][8-node slice][digits 0..3 | 4, 5 | 6], then the CTA's tiles of
   // outputs (blockIdx.y, + gridDim.y, ...): their K steps and exponents
   extern __shared__ __align__(16) unsigned char rm_smem[];
@@ -306,8 +324,13 @@ __global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const RmArgs a) 
       for (int i = 0; i < 4; ++i) {
         const int key = ek[ch][slice * 8 + 2 * t + (i & 1)];
         const int e = eo[(u * nch + ch) * 16 + g + 8 * (i >> 1)];
-        const int ee = (key >= 0x7ff00000 || e == 0x7fff ? kNonFinite : e) + key_exp(key);
-        const double v = few ? compose<true>(c[i], ee) : compose<false>(c[i], ee);
+        double v = 0.0;
+        if (key < 0x7ff00000 && e != 0x7fff) {
+          const int ee = e + key_exp(key);
+          v = few ? compose<true>(c[i], ee) : compose<false>(c[i], ee);
+        } else if (live(i)) {
+          v = rm_plain(&a, ch, a.obeg + u * 16 + g + 8 * (i >> 1), i0 + slice * 8 + 2 * t + (i & 1));
+        }
         x[i] = begun ? x[i] + v : v;
       }
       begun = true;
@@ -353,7 +376,7 @@ int recombine_mma(double* Xp, int64_t n, const double* Vbase, int64_t vstride, c
     const unsigned gy = std::max(1u, std::min<unsigned>((unsigned)(nt + 1) / 2, 304u / gx));
     const int smem = ks * kRmVStep + nt * (8 + 32 * ((ks + kChunkSteps - 1) / kChunkSteps));
     rm_gemm_kernel<<<dim3(gx, gy), kRmThreads, smem, st>>>(
-        RmArgs{Xp, n, Vbase, Z, Zp, W, list, rs.tiles, rs.exps, mask, ks, obeg_min, oend_max, rc.abort});
+        RmArgs{Xp, n, Vbase, Z, Zp, W, list, rs.tiles, rs.exps, mask, coef, ldo, ks, obeg_min, oend_max, rc.abort});
     launches += 2;
   }
   return launches;
