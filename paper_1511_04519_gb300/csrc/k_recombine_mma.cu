@@ -11,8 +11,13 @@
 //
 //   rm_list: the round's k in order of their columns' first outputs, so that
 //     16 consecutive ones (a K step) live on few outputs, each with the power of
-//     two that brings z' and z - w to the size of a basis vector (their largest
-//     entries, taken by krylov_start);
+//     two that brings its vector to the size of its column's response: a
+//     node's digits then start at the largest that any column has there, and an
+//     output's at the columns' relative size at that time.  The error is below
+//     2^-54 a term of the first times the second, so that small currents keep
+//     their digits beside large ones and a long tail its own (with the bare
+//     vectors, currents of 1e-12 of the largest lost half of their digits at the
+//     nodes where they act);
 //   rm_coef: per tile of 16 outputs the digits of the K steps that it meets,
 //     and the set of those (a 64-bit mask);
 //   rm_gemm: a CTA splits the vectors' values at its 32 nodes once, keeps the
@@ -52,7 +57,8 @@ constexpr int kRmMaxCh = kRmMaxSteps / kChunkSteps;
 // disagree with the recording; the run is then discarded) are empty.
 __global__ void __launch_bounds__(1024)
 rm_list_kernel(RoundCols rc, const int32_t* __restrict__ order, const int32_t* __restrict__ mcol,
-               const int32_t* __restrict__ tcut, const double* __restrict__ pbound, int K,
+               const int32_t* __restrict__ tcut, const double* __restrict__ beta,
+               const double* __restrict__ pbound, int K,
                int64_t vstride, int64_t gstride, int64_t n, RmK* __restrict__ list, int ktot, int kpad, unsigned long long* __restrict__ mask,
                int nmask) {
   __shared__ int warp_sum[32];
@@ -92,13 +98,16 @@ rm_list_kernel(RoundCols rc, const int32_t* __restrict__ order, const int32_t* _
       const int ov = tcut ? ob + tcut[2 * q] : oe;
       const int op = tcut && tcut[2 * q + 1] ? ov : oe;
       const int64_t vb = (int64_t)rc.vslot[q] * vstride, gb = (int64_t)rc.group[q] * gstride;
-      auto scale = [](double largest) {  // its binary exponent, 0 for zero, inf and NaN
-        const int e = (__double2hiint(largest) >> 20) & 0x7ff;
+      auto size = [](double x) {  // its binary exponent, 0 for zero, inf and NaN
+        const int e = (__double2hiint(x) >> 20) & 0x7ff;
         return e == 0 || e == 0x7ff ? 0 : e - 1022;
       };
-      for (int j = 0; j < m && k < ktot; ++j, ++k) list[k] = RmK{vb + (int64_t)j * n, q, j, ob, ov, 0, 0};
-      if (k < ktot) list[k++] = RmK{gb, q, kMaxM, ob, op, scale(pbound[2 * q + 1]), 0};
-      if (k < ktot) list[k++] = RmK{gb, q, kMaxM + 1, ob, op, scale(pbound[2 * q]), 0};
+      // the column's response: ||v|| V y, L z' and z - w; vectors of zeros stay out
+      const double zw = pbound[2 * q], zp = pbound[2 * q + 1];
+      const int sq = size(fmax(beta[q], fmax(zw, rc.len[q] * zp)));
+      for (int j = 0; j < m && k < ktot; ++j, ++k) list[k] = RmK{vb + (int64_t)j * n, q, j, ob, ov, -sq, 0};
+      if (k < ktot) list[k++] = RmK{zp == 0.0 ? -1 : gb, q, kMaxM, ob, op, size(zp) - sq, 0};
+      if (k < ktot) list[k++] = RmK{zw == 0.0 ? -1 : gb, q, kMaxM + 1, ob, op, size(zw) - sq, 0};
     }
     __syncthreads();
   }
@@ -204,7 +213,7 @@ __global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const __grid_con
   const int nch = (a.ksteps + kChunkSteps - 1) / kChunkSteps, ntile = (a.oend - a.obeg + 15) / 16;
   unsigned long long* mk = reinterpret_cast<unsigned long long*>(rm_smem + a.ksteps * kRmVStep);
   int16_t* eo = reinterpret_cast<int16_t*>(mk + ntile);
-  for (int i = threadIdx.x; i < kRmMaxCh * kRmNodes; i += kRmThreads) (&ek[0][0])[i] = 0;
+  for (int i = threadIdx.x; i < kRmMaxCh * kRmNodes; i += kRmThreads) (&ek[0][0])[i] = -kNonFinite;
   for (int i = threadIdx.x; i < ntile; i += kRmThreads) mk[i] = __ldg(a.mask + i);
   for (int i = threadIdx.x; i < ntile * nch * 8; i += kRmThreads)
     reinterpret_cast<int*>(eo)[i] = __ldg(reinterpret_cast<const int*>(a.exps) + i);
@@ -212,24 +221,28 @@ __global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const __grid_con
   // ---- the vectors' digits at the CTA's nodes: warp items (K step, slice), lane
   // node g of the slice, terms 2t, 2t + 1, 2t + 8, 2t + 9 (mma.sync's B operand)
   const int items = a.ksteps * (kRmNodes / 8);
-  auto load = [&](int it, double (&v)[4]) {
+  auto load = [&](int it, double (&v)[4], int (&sc)[4]) {
     const int ks = it / (kRmNodes / 8);
     const int64_t i = i0 + (it % (kRmNodes / 8)) * 8 + g;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const RmK e = a.list[ks * 16 + 2 * t + (u & 1) + (u >> 1) * 8];
       double x = 0.0;
-      if (e.off >= 0 && i < a.n) {
-        if (e.j < kMaxM) x = a.Vb[e.off + i];
-        else x = ldexp(e.j == kMaxM ? a.Zp[e.off + i] : a.Z[e.off + i] - a.W[e.off + i], -e.sc);
-      }
+      if (e.off >= 0 && i < a.n)
+        x = e.j < kMaxM ? a.Vb[e.off + i] : e.j == kMaxM ? a.Zp[e.off + i] : a.Z[e.off + i] - a.W[e.off + i];
       v[u] = x;
+      sc[u] = e.sc;
     }
   };
   for (int it = warp; it < items; it += kRmThreads / 32) {
     double v[4];
-    load(it, v);
-    int m = max(max(exp_key(v[0]), exp_key(v[1])), max(exp_key(v[2]), exp_key(v[3])));
+    int sc[4], m = -kNonFinite;
+    load(it, v, sc);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int key = exp_key(v[u]);
+      m = max(m, key >= 0x7ff00000 ? kNonFinite : key_exp(key) - sc[u]);
+    }
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
     if (t == 0)
@@ -238,11 +251,12 @@ __global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const __grid_con
   __syncthreads();
   for (int it = warp; it < items; it += kRmThreads / 32) {
     double v[4];
-    load(it, v);
-    const int e = key_exp(ek[it / (kRmNodes / 8) / kChunkSteps][(it % (kRmNodes / 8)) * 8 + g]);
+    int sc[4];
+    load(it, v, sc);
+    const int e = ek[it / (kRmNodes / 8) / kChunkSteps][(it % (kRmNodes / 8)) * 8 + g];
     uint64_t d[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) d[u] = digits(v[u], e);
+    for (int u = 0; u < 4; ++u) d[u] = digits(v[u], e + sc[u]);
     uint32_t b[kDigits];
 #pragma unroll
     for (int p = 0; p < kDigits; ++p) {
@@ -322,11 +336,11 @@ __global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const __grid_con
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int key = ek[ch][slice * 8 + 2 * t + (i & 1)];
+        const int en = ek[ch][slice * 8 + 2 * t + (i & 1)];  // a value's exponent, kNonFinite: an inf or NaN
         const int e = eo[(u * nch + ch) * 16 + g + 8 * (i >> 1)];
         double v = 0.0;
-        if (key < 0x7ff00000 && e != 0x7fff) {
-          const int ee = e + key_exp(key);
+        if (en < kNonFinite && e != 0x7fff) {
+          const int ee = e + en;
           v = few ? compose<true>(c[i], ee) : compose<false>(c[i], ee);
         } else if (live(i)) {
           v = rm_plain(&a, ch, a.obeg + u * 16 + g + 8 * (i >> 1), i0 + slice * 8 + 2 * t + (i & 1));
@@ -355,7 +369,7 @@ int recombine_mma(double* Xp, int64_t n, const double* Vbase, int64_t vstride, c
                   const double* Zp, const double* W, int64_t gstride, const RoundCols& rc,
                   const int32_t* order, const int32_t* mcol, const double* coef, int ldo, int K,
                   int kdim, int obeg_min, int oend_max, const RmScratch& rs, cudaStream_t st,
-                  const double* pbound, const int32_t* tcut) {
+                  const double* beta, const double* pbound, const int32_t* tcut) {
   const int nt = (oend_max - obeg_min + 15) / 16;
   if (K <= 0 || nt <= 0) return 0;
   const int ktot = kdim + 2 * K, steps = (ktot + 15) / 16;
@@ -363,7 +377,7 @@ int recombine_mma(double* Xp, int64_t n, const double* Vbase, int64_t vstride, c
   const int most = std::min(kRmMaxSteps, (kRmSmemMax - nt * (8 + 32 * kRmMaxCh)) / kRmVStep);
   const int parts = (steps + most - 1) / most;
   int launches = 1;
-  rm_list_kernel<<<1, 1024, 0, st>>>(rc, order, mcol, tcut, pbound, K, vstride, gstride, n, rs.list,
+  rm_list_kernel<<<1, 1024, 0, st>>>(rc, order, mcol, tcut, beta, pbound, K, vstride, gstride, n, rs.list,
                                      ktot, steps * 16, rs.mask, nt * parts);
   for (int p = 0; p < parts; ++p) {
     const int s0 = steps * p / parts, ks = steps * (p + 1) / parts - s0;

@@ -297,13 +297,14 @@ size_t rm_tiles_bytes(int n_times);
 size_t rm_exps(int n_times);
 bool rm_set_limits();
 // Xp[o][i] += the round's columns (V y and -P) at outputs [obeg_min, oend_max);
-// kdim = sum of mcol; order (or null): the columns by first output; pbound: the
-// columns' largest |z - w| and |z'| (krylov_start); tcut as recombine.  Returns the number of kernels launched.
+// kdim = sum of mcol; order (or null): the columns by first output; beta: the
+// columns' ||v||, pbound: their largest |z - w| and |z'| (krylov_start); tcut as
+// recombine.  Returns the number of kernels launched.
 int recombine_mma(double* Xp, int64_t n, const double* Vbase, int64_t vstride, const double* Z,
                   const double* Zp, const double* W, int64_t gstride, const RoundCols& rc,
                   const int32_t* order, const int32_t* mcol, const double* coef, int ldo, int K,
                   int kdim, int obeg_min, int oend_max, const RmScratch& rs, cudaStream_t st,
-                  const double* pbound, const int32_t* tcut);
+                  const double* beta, const double* pbound, const int32_t* tcut);
 // Where the tensor cores take a round: from 4 terms per output on average (the
 // FP64 kernel's time is the terms, about 2.5 ms per 180k nodes, 1,000 outputs and
 // 4 terms; the tensor cores' a tile's conversion and X, whatever the terms up to

@@ -1833,7 +1833,8 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
         nd * terms >= kRmMinWork) {
       rl = recombine_mma(c->Xp, n, c->Vb, vstride, c->Zb, c->Zpb, c->Wb, n, rc,
                          c->serial ? nullptr : c->rc_order + r.begin, c->ss.m, c->coef, c->n_times, K,
-                         kdim, r.obeg_min, r.oend_max, c->rm, st, c->pbound, teps > 0.0 ? c->tcut : nullptr);
+                         kdim, r.obeg_min, r.oend_max, c->rm, st, c->ss.beta, c->pbound,
+                         teps > 0.0 ? c->tcut : nullptr);
       if (teps == 0.0 && kdim >= kTcMinKdim && r.cover >= kTcMinCover) pc.tc_rounds++;
     } else {
       recombine(c->Xp, n, c->n_times, c->Vb, vstride, c->Zb, c->Zpb, c->Wb, n, rc, c->ss.m, c->coef,
