@@ -75,11 +75,12 @@ struct SmallShared {
   double ce[3][kMat];
 };
 
-// e^{hH} at t[0..count) into sh.ce, one worker each
+// e^{hH} at h = t[k] into sh.ce[k] for the k in want[0..count), one worker each
 template <class Team>
-__device__ void team_expm(const double* t, int count, int m, SmallShared<Team::kWorkers>& sh) {
+__device__ void team_expm(const double (&t)[3], const int (&want)[3], int count, int m,
+                          SmallShared<Team::kWorkers>& sh) {
   for (int i = Team::worker(); i < count; i += Team::kWorkers)
-    expm_dev<typename Team::W>(sh.H, t[i], sh.ce[i], m, sh.w[Team::worker()]);
+    expm_dev<typename Team::W>(sh.H, t[want[i]], sh.ce[want[i]], m, sh.w[Team::worker()]);
   Team::G::sync();
 }
 
@@ -114,7 +115,8 @@ __device__ int residual_column(SmallState ss, const RoundCols& rc, int q, int j,
     rational_H<G>(Ht, m, gamma, sh.H, sh.w[0], ss.krylov);
     const double L = rc.len[q];
     const double t[3] = {fmin(rc.hfirst[q], L), L, dt};
-    team_expm<Team>(t, dt > 0.0 && Team::kWorkers > 2 ? 3 : 2, m, sh);
+    const int all[3] = {0, 1, 2};
+    team_expm<Team>(t, all, dt > 0.0 && Team::kWorkers > 2 ? 3 : 2, m, sh);
     if (G::rank() == 0) {
       // r = ||v|| |s h_{m+1,m} e_m^T e^{hH} e_1|, s making h_{m+1,m} dimensionless
       const double c = ss.beta[q] * fabs(ss.rscale * Ht[m * kMaxM + (m - 1)]);
@@ -159,12 +161,16 @@ __device__ void coef_column(SmallState ss, const RoundCols& rc, int q, double ga
     const double* Ht = ss.Ht + (int64_t)q * kMaxB * kMaxM;
     const double beta = ss.beta[q];
     const double hf = rc.hfirst[q], L = rc.len[q];
-    // the exponentials of the residual test of this m when it took them
-    if (sh.cm != m || sh.ch[1] != L || (no > 0 && sh.ch[0] != hf) || (no > 1 && sh.ch[2] != dt_out)) {
-      if (sh.cm != m) rational_H<G>(Ht, m, gamma, sh.H, sh.w[0], ss.krylov);
-      const double t[3] = {no > 0 ? hf : L, L, dt_out};
-      team_expm<Team>(t, no > 1 ? 3 : 2, m, sh);
-    }
+    // at the first output, the segment's end and the output interval, without
+    // those that the residual test of this m took
+    const bool have = sh.cm == m;
+    const double t[3] = {hf, L, dt_out};
+    int want[3], count = 0;
+    if (no > 0 && !(have && sh.ch[0] == hf)) want[count++] = 0;
+    if (!(have && sh.ch[1] == L)) want[count++] = 1;
+    if (no > 1 && !(have && sh.ch[2] == dt_out)) want[count++] = 2;
+    if (!have) rational_H<G>(Ht, m, gamma, sh.H, sh.w[0], ss.krylov);
+    team_expm<Team>(t, want, count, m, sh);
     for (int i = G::rank(); i < m; i += G::size()) {
       yend[(int64_t)q * kMaxM + i] = beta * sh.ce[1][i * kLd];
       if (no > 0) cq[i] = beta * sh.ce[0][i * kLd];
