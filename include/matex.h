@@ -122,12 +122,14 @@ typedef struct matex_opts {
                               solutions, Arnoldi with its residual test, output coefficients,
                               next state) in one CTA, both triangular substitutions level by
                               level in its shared memory; only the recombination is a launch of
-                              its own.  Possible when n <= 8192 (and 16 n + 34 KB fit one CTA's
-                              shared memory), krylov 0 or 1, tape 0 and tail_eps 0; 2 returns
-                              MATEX_ERR_ARG otherwise.  With 0 the setup times one such solve
-                              pair against the batched path's single-column pair and takes the
-                              resident rounds when they are at most twice as long (they also
-                              replace the ~12 other launches of every Arnoldi step).  The
+                              its own.  Possible when n <= 8192 (and 16 n + 36 KB and the plan
+                              fit one CTA's shared memory: about 3,000 nodes), krylov 0 or 1,
+                              tape 0 and tail_eps 0; 2 returns MATEX_ERR_ARG otherwise.  With 0
+                              the setup compares them with the batched rounds: by one solve pair
+                              each where that decides, else by the time of the context's own
+                              first rounds.  Where the batched rounds win, a run whose new
+                              currents or capacitances change the recorded Krylov dimensions
+                              takes the resident ones (matex_stats.resident of that run).  The
                               input solutions of every segment (sources only) are solved ahead
                               of the rounds in one launch when they fit a quarter of the free
                               memory; 3: as 2, but each round kernel solves its own (the path
@@ -182,7 +184,8 @@ typedef struct matex_stats {
   int32_t tc_rounds;       /* dense segment rounds of the last exact run on the tensor cores: at
                               least 16 basis vectors, whose columns hold at least a quarter of
                               the round's outputs (sparser rounds may run there too) */
-  int32_t resident;        /* 1: the segment rounds run as resident rounds (opts.resident) */
+  int32_t resident;        /* 1: the segment rounds run as resident rounds (opts.resident; at
+                              setup the choice, after a run what it took) */
   int32_t tc_solve_supernodes;  /* supernodes at least tc_min_width wide whose solve products
                                    can run on the tensor cores (0: none or tc_solve off) */
   int32_t tc_solve_min_cols;    /* smallest column count at which they do (0: never) */

@@ -81,20 +81,28 @@ struct matex_ctx {
   Symbolic SC;                     // S in larger supernodes, for the tensor-core solves
   std::vector<LevelPlan> levels;
   SplitScratch split;              // chunked reductions of the level launches
-  // resident rounds (opts.resident): per-level work lists, the choice, and
-  // the setup's timings of one solve pair both ways (ms, -1 if not taken)
   // level solves on the tensor cores (opts.tc_solve, k_sptrsv_mma.cu): plan,
   // panel digits, and per column count whether a solve takes them
   MmPlan mm;
   double* mm_pan = nullptr;  // a factor's panels on their way into digits
   bool mm_ok = false;
   std::vector<int8_t> mm_by_ncols;
+  // resident rounds (opts.resident): per-level work lists, the factors' resident
+  // copies, the choice, and the setup's timings of one solve pair both ways
+  // (ms, -1 if not taken)
   ResidentPlan rplan;
-  ResFactor rM, rG;          // the factors' resident copies
+  ResFactor rM, rG;
   ResStoreSup* rsup = nullptr;
   bool resident_ok = false;  // plan built and shared-memory limits set
   bool resident = false;
   float res_pair_ms = -1.f, lvl_pair_ms = -1.f;
+  int timed_rounds = 0;      // > 0: run_pass takes that many rounds, for their time alone
+  bool timed_again = false;  // and the resident rounds' input solves are there
+  // batched rounds chosen where resident ones fit too: runs with new currents or
+  // capacitances may take those (run_device)
+  bool res_new = false;      // they may
+  bool new_inputs = false;   // some were set since the last run
+  bool drifts = false;       // new ones have changed the recorded counts before
   // resident rounds: every column record's z' and w, solved ahead of the
   // rounds in one launch per run (null: each round kernel solves its own)
   double *pre_zp = nullptr, *pre_w = nullptr;
@@ -857,6 +865,29 @@ int solve_cols(matex_ctx* c, const DevFactor& F, int ncols);
 
 std::string tune_key(matex_ctx* c);
 
+// A yes/no choice of an earlier setup in the MATEX_AUTOTUNE_CACHE file (-1: none), and its entry.
+int cached_choice(const std::string& key) {
+  const char* cache = std::getenv("MATEX_AUTOTUNE_CACHE");
+  FILE* f = cache ? std::fopen(cache, "r") : nullptr;
+  if (!f) return -1;
+  char line[1024];
+  int found = -1;
+  while (std::fgets(line, sizeof(line), f)) {
+    const std::string l(line);
+    if (l.compare(0, key.size() + 1, key + " ") == 0 && l.size() > key.size() + 1)
+      found = l[key.size() + 1] == '1' ? 1 : 0;
+  }
+  std::fclose(f);
+  return found;
+}
+void store_choice(const std::string& key, bool choice) {
+  const char* cache = std::getenv("MATEX_AUTOTUNE_CACHE");
+  if (FILE* f = cache ? std::fopen(cache, "a") : nullptr) {
+    std::fprintf(f, "%s %d\n", key.c_str(), choice ? 1 : 0);
+    std::fclose(f);
+  }
+}
+
 // opts.single_column 2: the single-column kernels for every solve of one
 // column; 0 (with the tuned launch mode): where their solve pair is at least
 // 5 % faster than the tuned path's (best of three after a warm-up each),
@@ -868,23 +899,11 @@ void autotune_k1(matex_ctx* c) {
     c->k1_use = true;
     return;
   }
-  const char* cache = std::getenv("MATEX_AUTOTUNE_CACHE");
   const std::string key = "k1:" + tune_key(c);
-  if (cache) {
-    if (FILE* f = std::fopen(cache, "r")) {
-      char line[1024];
-      int found = -1;
-      while (std::fgets(line, sizeof(line), f)) {
-        const std::string l(line);
-        if (l.compare(0, key.size() + 1, key + " ") == 0 && l.size() > key.size() + 1)
-          found = l[key.size() + 1] == '1' ? 1 : 0;
-      }
-      std::fclose(f);
-      if (found >= 0) {
-        c->k1_use = found == 1;
-        return;
-      }
-    }
+  const int found = cached_choice(key);
+  if (found >= 0) {
+    c->k1_use = found == 1;
+    return;
   }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -908,12 +927,7 @@ void autotune_k1(matex_ctx* c) {
   c->k1_use = cudaGetLastError() == cudaSuccess && mine < 0.95f * ref;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (cache) {
-    if (FILE* f = std::fopen(cache, "a")) {
-      std::fprintf(f, "%s %d\n", key.c_str(), c->k1_use ? 1 : 0);
-      std::fclose(f);
-    }
-  }
+  store_choice(key, c->k1_use);
 }
 
 // Tensor-core level solves (k_sptrsv_mma.cu): per direction the supernodes by
@@ -1116,23 +1130,11 @@ void choose_mm(matex_ctx* c) {
   }
   c->mm_by_ncols[1] = 0;
   if (c->opts.single_column != 0 || c->opts.solve_mode != 2) return;
-  const char* cache = std::getenv("MATEX_AUTOTUNE_CACHE");
   const std::string key = "mm1:" + tune_key(c);
-  if (cache) {
-    if (FILE* f = std::fopen(cache, "r")) {
-      char line[1024];
-      int found = -1;
-      while (std::fgets(line, sizeof(line), f)) {
-        const std::string l(line);
-        if (l.compare(0, key.size() + 1, key + " ") == 0 && l.size() > key.size() + 1)
-          found = l[key.size() + 1] == '1' ? 1 : 0;
-      }
-      std::fclose(f);
-      if (found >= 0) {
-        c->mm_by_ncols[1] = (int8_t)found;
-        return;
-      }
-    }
+  const int found = cached_choice(key);
+  if (found >= 0) {
+    c->mm_by_ncols[1] = (int8_t)found;
+    return;
   }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -1154,12 +1156,7 @@ void choose_mm(matex_ctx* c) {
   c->mm_by_ncols[1] = cudaGetLastError() == cudaSuccess && best[1] < 0.95f * best[0];
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (cache) {
-    if (FILE* f = std::fopen(cache, "a")) {
-      std::fprintf(f, "%s %d\n", key.c_str(), (int)c->mm_by_ncols[1]);
-      std::fclose(f);
-    }
-  }
+  store_choice(key, c->mm_by_ncols[1] != 0);
 }
 
 int solve_cols(matex_ctx* c, const DevFactor& F, int ncols) {
@@ -1601,7 +1598,9 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
     launches += nl;
   };
   // constant part: x_dc = G^{-1} dc_inject
-  if (c->opts.include_dc && c->dc_perm) {
+  if (c->timed_rounds) {
+    // the rounds alone
+  } else if (c->opts.include_dc && c->dc_perm) {
     e = prof_begin(c);
     gather_cols(c->Y, c->ldy, 1, c->dc_perm, 0, nullptr, nullptr, nullptr, n, st);
     moved(e, 1, 1, false);
@@ -1631,10 +1630,11 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
   }
   matex_status s = MATEX_OK;
   const std::vector<Round>& rounds = c->serial ? c->serial_rounds : c->rounds;
-  const size_t nbatch = c->serial ? 1 : c->batches.size();
+  const size_t nbatch = c->serial || c->timed_rounds ? 1 : c->batches.size();
   for (size_t bi = 0; bi < nbatch; ++bi) {
   const int r0 = c->serial ? 0 : c->batches[bi].r0;
-  const int r1 = c->serial ? (int)rounds.size() : c->batches[bi].r1;
+  int r1 = c->serial ? (int)rounds.size() : c->batches[bi].r1;
+  if (c->timed_rounds) r1 = std::min(r1, r0 + c->timed_rounds);
   const int i0 = c->serial ? 0 : c->batches[bi].i0;
   const int ng = c->serial ? (int)c->init_groups.size() : c->batches[bi].ni;
   if (bi > 0) {
@@ -1679,7 +1679,7 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
     }
     return ra;
   };
-  if (c->resident && c->pre_zp && bi == 0) {
+  if (c->resident && c->pre_zp && bi == 0 && !c->timed_again) {
     // the input solves of every column record (sources only, no state): one
     // launch, one CTA per record, instead of two solves in each round kernel
     Round all;
@@ -1928,6 +1928,7 @@ matex_status finish_run(matex_ctx* c, const PassCounts& pc, double t0, bool repl
   }
   o.sweeps_M = pc.sweepsM;
   o.tc_rounds = pc.tc_rounds;
+  o.resident = c->resident ? 1 : 0;
   o.sweeps_G = pc.sweepsG;
   o.solve_columns = pc.solve_cols;
   if (c->resident) {
@@ -1970,9 +1971,33 @@ matex_status replay_flags(matex_ctx* c, bool* diverged) {
   return MATEX_OK;
 }
 
+// One run on resident rounds, plainly launched (nothing is read back between
+// them), by a context whose choice are the batched ones; their recording stays.
+matex_status run_resident_once(matex_ctx* c, double* x_out, double t0, matex_stats* stats) {
+  c->resident = true;
+  PassCounts pc;
+  int tmp = 0;
+  matex_status s = run_pass(c, false, pc);
+  if (s == MATEX_OK) {
+    permute_out(x_out, c->Xp, c->out_map, c->nrows_out, c->n, c->n_times, c->st);
+    s = read_count(c, &tmp);
+  }
+  if (s == MATEX_OK) s = cuda_check(c, "resident run");
+  if (s == MATEX_OK) s = finish_run(c, pc, t0, false, stats);
+  c->resident = false;
+  return s;
+}
+
 matex_status run_device(matex_ctx* c, double* x_out, matex_stats* stats) {
   const double t0 = now_ms();
   matex_status s;
+  // New inputs mostly change some column's Krylov dimension: the replay is
+  // then lost, and a plain run (the host reads every count) with a new recording
+  // takes two to three replays' time.  Where the resident rounds fit, which hold
+  // no counts, they serve that run, and from then on every run with new inputs.
+  const bool fresh = c->new_inputs && c->res_new && graph_allowed(c);
+  c->new_inputs = false;
+  if (fresh && c->drifts) return run_resident_once(c, x_out, t0, stats);
   if (graph_allowed(c) && c->gexec) {
     if (cudaGraphLaunch(c->gexec, c->st) != cudaSuccess) return cuda_check(c, "graph launch");
     permute_out(x_out, c->Xp, c->out_map, c->nrows_out, c->n, c->n_times, c->st);
@@ -1980,6 +2005,10 @@ matex_status run_device(matex_ctx* c, double* x_out, matex_stats* stats) {
     bool diverged = false;
     if ((s = replay_flags(c, &diverged)) != MATEX_OK) return s;
     if (!diverged) return finish_run(c, c->graph_counts, t0, true, stats);
+    if (fresh) {
+      c->drifts = true;
+      return run_resident_once(c, x_out, t0, stats);
+    }
     drop_graph(c);  // the counts changed: run plainly and record again
   }
   c->kit_trace.clear();
@@ -1996,6 +2025,78 @@ matex_status run_device(matex_ctx* c, double* x_out, matex_stats* stats) {
   }
   if (graph_allowed(c)) capture_graph(c);
   return finish_run(c, pc, t0, false, stats);
+}
+
+// The rounds that a setup times: rise, fall and what follows, for most columns.
+constexpr int kTimedRounds = 3;
+
+// Time (ms) of the first kTimedRounds rounds as a run has them, resident or
+// batched as c->resident says, the better of two; < 0 when they failed.  Batched
+// rounds as replays of their recording (unless graphs are off); resident ones
+// plainly, as nothing is read back between them, without the input solves ahead.
+float time_rounds(matex_ctx* c) {
+  c->timed_rounds = kTimedRounds;
+  c->kit_trace.clear();
+  PassCounts pc;
+  bool ok = run_pass(c, false, pc) == MATEX_OK;
+  c->timed_again = true;
+  if (ok && c->opts.graph && !c->resident) {
+    capture_graph(c);
+    ok = c->gexec != nullptr;
+  }
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  float best = -1.f;
+  for (int rep = 0; ok && rep < 2; ++rep) {
+    float ms = 0.f;
+    cudaEventRecord(e0, c->st);
+    ok = c->gexec ? cudaGraphLaunch(c->gexec, c->st) == cudaSuccess : run_pass(c, false, pc) == MATEX_OK;
+    cudaEventRecord(e1, c->st);
+    ok = cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ok;
+    best = best < 0.f ? ms : std::min(best, ms);
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  drop_graph(c);
+  c->kit_trace.clear();
+  c->graph_gen = 0;
+  c->graph_ms = 0.0;
+  c->timed_rounds = 0;
+  c->timed_again = false;
+  return ok && cudaGetLastError() == cudaSuccess ? best : -1.f;
+}
+
+// Whether the rounds run resident, where they fit.  A resident solve pair (one
+// CTA) up to 1.6 times as long as the batched path's: yes, the resident rounds
+// have no launches between their steps (grids of 600 to 1,600 nodes, ratios of 1.0
+// to 1.6: 0.3 to 0.8 of the batched runs' time).  Above 4: no (none fits).  Between, by
+// what the run's own rounds take: at 2,000 to 3,000 nodes, ratios of 1.9 to 3, the
+// resident run takes 0.6 to 1.4 times the batched one's, the less the fewer
+// columns.  Ties go to the resident rounds, whose results are reproducible and
+// whose time is the same with new currents.
+bool choose_resident(matex_ctx* c) {
+  const double ratio = (double)c->res_pair_ms / (double)c->lvl_pair_ms;
+  if (!(ratio > 1.6) || ratio > 4.0 || c->rounds.empty()) return !(ratio > 4.0);
+  char shape[96];
+  std::snprintf(shape, sizeof(shape), ";k=%d;rounds=%d;rec=%lld;t=%d;g=%d", c->Kmax, (int)c->rounds.size(),
+                (long long)c->n_records, c->n_times, c->opts.graph);
+  const std::string key = "res:" + tune_key(c) + shape;
+  const int found = cached_choice(key);
+  if (found >= 0) return found == 1;
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  const int timed = std::min(kTimedRounds, c->batches[0].r1 - c->batches[0].r0);
+  const double f = (double)c->rounds.size() / std::max(1, timed);
+  const double ahead = c->pre_zp ? 2.0 * c->res_pair_ms * (double)((c->n_records + sms - 1) / sms) : 0.0;
+  c->resident = true;
+  const double res = time_rounds(c);
+  c->resident = false;
+  const double bat = time_rounds(c);
+  if (res < 0.0 || bat < 0.0) return false;
+  const bool yes = f * res + ahead <= 1.05 * f * bat;
+  store_choice(key, yes);
+  return yes;
 }
 
 // Reverse of the columns [qa, qa + K) of round r, given their tape entries
@@ -2831,7 +2932,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   }
   if (o.resident != 1 && o.krylov != 2 && o.tape == 0 && o.tail_eps == 0.0 &&
       n <= kResidentMaxN) {
-    // resident rounds: one CTA's solve pair against the batched path's
+    // resident rounds: one CTA's solve pair and the batched path's
     // single-column pair (in its tuned launch mode), best of five each
     if (plan_resident(c, kResidentThreads) && resident_fits(n, c->rplan) &&
         resident_set_limits(n, c->rplan)) {
@@ -2857,17 +2958,18 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
       c->lvl_pair_ms = best;
-      c->resident = c->res_pair_ms > 0.f && (o.resident >= 2 || c->res_pair_ms <= 2.f * best);
       // room for every record's z' and w (at most a quarter of the free
       // memory): the input solves then run ahead of the rounds (not with
       // resident = 3, which keeps them in the round kernels)
       size_t free_b = 0, total_b = 0;
       cudaMemGetInfo(&free_b, &total_b);
       const double need = 16.0 * (double)c->n_records * (double)n;
-      if (c->resident && o.resident != 3 && c->n_records > 0 && need <= 0.25 * (double)free_b &&
+      if (c->res_pair_ms > 0.f && o.resident != 3 && c->n_records > 0 && need <= 0.25 * (double)free_b &&
           !(c->alloc(c->pre_zp, (size_t)c->n_records * n) &&
             c->alloc(c->pre_w, (size_t)c->n_records * n)))
         c->pre_zp = c->pre_w = nullptr;
+      c->resident = c->res_pair_ms > 0.f && (o.resident >= 2 || choose_resident(c));
+      c->res_new = c->res_pair_ms > 0.f && !c->resident;
     }
     cudaGetLastError();
   }
@@ -2937,6 +3039,7 @@ matex_status matex_set_caps(matex_ctx* c, const double* cap) {
   }
   c->c_host.assign(cap, cap + c->n);
   c->taped = false;
+  c->new_inputs = true;
   c->tr_h = 0.0;  // the trapezoidal factor C + h/2 G is refactored on its next use
   c->setup_stats.setup_factor_ms = now_ms() - t;
   return MATEX_OK;
@@ -2981,6 +3084,7 @@ matex_status matex_set_sources(matex_ctx* c, const double* pwl_v_host) {
   cudaMemcpyAsync(c->pwl_v_d, pwl_v_host, sizeof(double) * c->pwl_v_host_shape.size(),
                   cudaMemcpyHostToDevice, c->st);
   c->taped = false;
+  c->new_inputs = true;
   return cuda_check(c, "set_sources");
 }
 
@@ -2996,6 +3100,7 @@ matex_status matex_run_host(matex_ctx* c, const double* pwl_v_host, double* x_ou
     if (cs != MATEX_OK) return cs;
     cudaMemcpyAsync(c->pwl_v_d, pwl_v_host, sizeof(double) * c->pwl_v_host_shape.size(),
                     cudaMemcpyHostToDevice, c->st);
+    c->new_inputs = true;
   }
   // Page-locked host output: the final permutation kernel writes the voltages
   // straight into host memory through its device mapping (over NVLink-C2C on
@@ -3783,6 +3888,7 @@ matex_status batch_fail(matex_batch* b, matex_status s, const std::string& m) {
 matex_status batch_record(matex_batch* b, matex_ctx* c) {
   if (!c->out_buf && !c->alloc(c->out_buf, (size_t)c->n_times * c->nrows_out))
     return batch_fail(b, MATEX_ERR_OOM, "output buffer");
+  c->new_inputs = false;  // to be recorded
   matex_status s = run_device(c, c->out_buf, nullptr);
   if (s != MATEX_OK && s != MATEX_ERR_NOCONV) return batch_fail(b, s, c->err);
   if (!c->graph) return batch_fail(b, MATEX_ERR_CUDA, "a context's run could not be recorded as a graph");
@@ -3896,6 +4002,7 @@ matex_status matex_batch_run(matex_batch* b, double* const* x_outs, matex_stats*
     if (c->h_count[1] != 0)
       return batch_fail(b, MATEX_ERR_TIMEOUT, "a bounded wait of the persistent solve expired");
     matex_stats* si = stats ? stats + i : nullptr;
+    c->new_inputs = false;
     if (c->h_count[2] != 0) {
       // this grid's counts diverged from its recording: redo it plainly
       drop_graph(c);
