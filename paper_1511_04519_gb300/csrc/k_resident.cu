@@ -21,7 +21,7 @@ namespace {
 
 
 // Norm of a vector whose squares' sums the threads hold, and its reciprocal (0
-// for a norm up to `least`), returned to every thread.  red: 32 doubles of
+// for a norm up to `least` or a NaN, as gs_scale_kernel has it), returned to every thread.  red: 32 doubles of
 // shared memory.  One warp adds the warps' sums and one thread takes the root
 // and the quotient: an FP64 instruction costs the CTA 64 clocks per four warps,
 // a division of all 512 threads 2,550 (measured).
@@ -40,7 +40,7 @@ __device__ __forceinline__ ResNorm res_block_norm(double v, double least, double
     if (threadIdx.x == 0) {
       const double r = sqrt(s);
       red[30] = r;
-      red[31] = r <= least ? 0.0 : 1.0 / r;
+      red[31] = r > least ? 1.0 / r : 0.0;
     }
   }
   __syncthreads();
@@ -356,14 +356,15 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_round_kernel(Res
   double* Ht = ss.Ht + (int64_t)q * kMaxB * kMaxM;
   for (int e = tid; e < kMaxB * kMaxM; e += nt) Ht[e] = 0.0;
   const bool quiet = beta <= 1e-300;
+  const double sc = beta != beta ? beta : nb.inv;  // a NaN stays one, as in start_finish_kernel
   if (tid == 0) {
     ss.beta[q] = beta;
     ss.m[q] = 0;
     ss.status[q] = quiet ? 4 : 0;
-    ss.scale[q] = nb.inv;
+    ss.scale[q] = sc;
   }
   if (!quiet) {
-    for (int64_t i = tid; i < n; i += nt) V[i] = b[i] * nb.inv;
+    for (int64_t i = tid; i < n; i += nt) V[i] = b[i] * sc;
     for (int j = 0; j < a.m_max; ++j) {
       // w = X1^{-1} C v_j (Alg. 1 with X2 = C)
       const double* __restrict__ vj = V + (int64_t)j * n;
