@@ -53,8 +53,9 @@ typedef enum matex_status {
 
 /* Options of matex_setup.  Start from matex_default_opts(). */
 typedef struct matex_opts {
-  int32_t col_block;       /* column block of the triangular solves: 0 = tuned per tree level,
-                              else 1, 2, 4 or 8 for every level */
+  int32_t col_block;       /* column block of the FP64 level solves: 0 = tuned per tree level,
+                              else 1, 2, 4 or 8 for every level (no effect on the solves that
+                              tc_solve puts on the tensor cores) */
   int32_t group_select;    /* -1: all groups; g >= 0: simulate only group g */
   int32_t include_dc;      /* 1: add the pads' constant DC state x_dc = G^{-1} dc_inject */
   int32_t n_rows;          /* 0: output every node; else the number of rows in `rows` */
@@ -140,8 +141,8 @@ typedef struct matex_opts {
                               every column count.  An error-free split of the FP64 operands into
                               seven 8-bit digits (error no larger than an FP64 dot product's),
                               one launch per tree level and direction (solve_mode 1 and 2) */
-  int32_t tc_min_width;    /* 0 (default): 64; else at least 32: the width from which
-                              tc_solve_supernodes counts */
+  int32_t tc_min_width;    /* 0, or at least 32: accepted as ever, without effect (every
+                              supernode's products run where tc_solve says) */
   int32_t single_column;   /* solves of one right-hand side: 0 (default) chosen at setup, 1 off,
                               2 on.  The single-column level kernels run one launch per tree level
                               and direction like the level launches, with everything that does
@@ -181,13 +182,12 @@ typedef struct matex_stats {
   int32_t tape_block;      /*   block as set up (0 otherwise) */
   int64_t tape_bytes;      /* device bytes of the adjoint's tape (tape 1) or of its checkpoints,
                               window tape and reverse work buffers (tape 2) */
-  int32_t tc_rounds;       /* dense segment rounds of the last exact run on the tensor cores: at
-                              least 16 basis vectors, whose columns hold at least a quarter of
-                              the round's outputs (sparser rounds may run there too) */
+  int32_t tc_rounds;       /* segment rounds of the last run whose recombination ran on the
+                              tensor cores */
   int32_t resident;        /* 1: the segment rounds run as resident rounds (opts.resident; at
                               setup the choice, after a run what it took) */
-  int32_t tc_solve_supernodes;  /* supernodes at least tc_min_width wide whose solve products
-                                   can run on the tensor cores (0: none or tc_solve off) */
+  int32_t tc_solve_supernodes;  /* supernodes of the tensor-core solves' plan, all of whose
+                                   products run there (0: no plan, or tc_solve off) */
   int32_t tc_solve_min_cols;    /* smallest column count at which they do (0: never) */
   int32_t single_column;        /* 1: single-column solves run the single-column level kernels */
 } matex_stats;

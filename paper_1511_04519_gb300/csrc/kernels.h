@@ -312,8 +312,6 @@ int recombine_mma(double* Xp, int64_t n, const double* Vbase, int64_t vstride, c
 // 23.4 at 16, 25.3 with the FP64 kernel alone.  Below 2e6 products the FP64
 // kernel takes less than the three launches.
 constexpr double kRmDensity = 4.0, kRmMinWork = 2e6;
-constexpr int kTcMinKdim = 16;         // a round counts as dense from this many basis vectors
-constexpr double kTcMinCover = 0.25;   // and this share of its (column, output) pairs held
 
 // Adjoint checkpoints: CK[q] = {X[groups[q]], Z[groups[q]]} ([K][2][n]), or the
 // reverse copy when restore is set (X, Z per group, [G][n]).

@@ -45,8 +45,7 @@ struct Round {
   int32_t begin;  // first column record
   int32_t K;      // columns
   int32_t obeg_min, oend_max;
-  double cover = 0.0;          // share of (column, output) pairs of the range the columns hold
-  double held = 0.0;           // those pairs
+  double held = 0.0;           // (column, output) pairs that the columns hold
 };
 
 // Device address of the allocation-free solve's static scratch array on
@@ -1835,7 +1834,7 @@ matex_status run_pass(matex_ctx* c, bool capture, PassCounts& pc) {
                          c->serial ? nullptr : c->rc_order + r.begin, c->ss.m, c->coef, c->n_times, K,
                          kdim, r.obeg_min, r.oend_max, c->rm, st, c->ss.beta, c->pbound,
                          teps > 0.0 ? c->tcut : nullptr);
-      if (teps == 0.0 && kdim >= kTcMinKdim && r.cover >= kTcMinCover) pc.tc_rounds++;
+      pc.tc_rounds++;
     } else {
       recombine(c->Xp, n, c->n_times, c->Vb, vstride, c->Zb, c->Zpb, c->Wb, n, rc, c->ss.m, c->coef,
                 c->n_times, K, r.obeg_min, r.oend_max, c->dt_out, st,
@@ -2692,9 +2691,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
       order_h[rd.begin + q] = q;
     }
     c->round_cover.push_back(cnt);
-    const int span = rd.oend_max - rd.obeg_min;
     rd.held = held;
-    rd.cover = span > 0 ? held / ((double)rd.K * span) : 0.0;
     std::stable_sort(order_h.begin() + rd.begin, order_h.begin() + rd.begin + rd.K,
                      [&](int32_t a, int32_t b) { return h_obeg[rd.begin + a] < h_obeg[rd.begin + b]; });
   }
@@ -2925,9 +2922,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
     cudaGetLastError();
   }
   if (c->mm_ok) {
-    const int minw = o.tc_min_width > 0 ? o.tc_min_width : 64;
-    for (int32_t s = 0; s < S.nsup; ++s)
-      c->setup_stats.tc_solve_supernodes += S.sup_first[s + 1] - S.sup_first[s] >= minw;
+    c->setup_stats.tc_solve_supernodes = c->mm.nsup;
     c->setup_stats.tc_solve_min_cols = c->mm_by_ncols[1] ? 1 : 2;
   }
   if (o.resident != 1 && o.krylov != 2 && o.tape == 0 && o.tail_eps == 0.0 &&
