@@ -103,10 +103,13 @@ typedef struct matex_opts {
   int32_t tape_block;      /* tape = 2: groups recomputed together (columns of the recompute
                               and reverse launches); 0 (default): chosen at setup */
   int32_t recombine;       /* the recombination (Eq. 6 at the outputs): 0 (default) on the
-                              tensor cores where enough terms meet in an output, as an
-                              error-free split of the FP64 operands into seven 8-bit digits
-                              whose products the FP32 accumulators hold exactly (error no
-                              larger than an FP64 dot product's); 1: FP64 FMAs only */
+                              tensor cores where enough terms meet in an output, each operand
+                              split into seven 8-bit digits whose products the FP32
+                              accumulators hold exactly.  The digits start at the largest
+                              value, over 128 terms, that a column's response takes at a node
+                              and at the columns' largest relative size at an output; the error
+                              is below 2^-53 a term of those two's product (an FP64 sum's: of
+                              the terms' own sizes).  1: FP64 FMAs only */
   int32_t decompose;       /* 0 (default): the groups as given (Sec. 3.1's bump groups);
                               1: every group's input is split further into single ramps: on
                               [0, T] a source is its value at t = 0 plus, at each of its
@@ -138,9 +141,14 @@ typedef struct matex_opts {
   int32_t tc_solve;        /* the level solves' dense products (P_s b_s forward, P_s^T [..]
                               backward) on the tensor cores: 0 (default) for two columns and
                               more, and for one where the setup times it faster; 1 off; 2 for
-                              every column count.  An error-free split of the FP64 operands into
-                              seven 8-bit digits (error no larger than an FP64 dot product's),
-                              one launch per tree level and direction (solve_mode 1 and 2) */
+                              every column count.  The operands are split into seven 8-bit
+                              digits, from the largest entry of a panel row and of a right-hand
+                              side over 128 terms down: a product is off by 2^-53 a term of
+                              those two's product at most (an FP64 dot product: of the terms
+                              themselves), so a solution is as accurate as the FP64 kernels'
+                              relative to its largest entry, while an entry 2^-k below the
+                              largest nearby may lose k digits, which the FP64 kernels keep.
+                              One launch per tree level and direction (solve_mode 1 and 2) */
   int32_t tc_min_width;    /* 0, or at least 32: accepted as ever, without effect (every
                               supernode's products run where tc_solve says) */
   int32_t single_column;   /* solves of one right-hand side: 0 (default) chosen at setup, 1 off,

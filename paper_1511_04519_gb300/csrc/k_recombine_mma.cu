@@ -1,11 +1,11 @@
-// FP64-accurate basis recombination on the tensor cores: the final step of
+// Basis recombination on the tensor cores: the final step of
 // Alg. 1 at every output of a segment round (Alg. 2's snapshots) and the sum of
 // the groups' responses,
 //   X[o][i] += sum over the round's columns q whose segment holds o of
 //              V_q y_q(o) + (z_q - w_q) + (t_o - l_q) z'_q            (Eq. 6),
 // as one contraction over k: a column's m basis vectors with the coefficients
 // y_q(o), z'_q with t_o - l_q and z_q - w_q with 1, each zero where the column
-// does not hold o.  Digit products of an error-free split (split8.cuh) on
+// does not hold o.  Digit products of a 54-bit split (split8.cuh) on
 // mma.sync: 16 outputs x 8 nodes over 16 terms take the FP64 pipe 1,024 clocks
 // of an SM, the 34 digit products 68.
 //

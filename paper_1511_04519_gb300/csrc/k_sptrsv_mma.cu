@@ -3,7 +3,8 @@
 // solves of Eq. 5/6),
 //   forward : [y_s; u_R] = P_s b_s, then b_R -= u_R (FP64 atomics),
 //   backward: x_s = P_s^T [D_s^{-1} y_s; -x_R],
-// as FP16 digit products (34 per tile) with the accuracy of FP64
+// as FP16 digit products (34 per tile), as accurate as FP64 relative to the
+// largest entries of a panel row and of a right-hand side over 128 terms
 // (split8.cuh).  The FP64 pipe (two FMA per clock and SM on GB300) bounds
 // k_sptrsv.cu: 8 panel rows x 16 right-hand sides over 16 terms take it 1,024
 // clocks of an SM, the 34 digit products of the same tile take mma.sync 68

@@ -1,5 +1,7 @@
-// Error-free split of FP64 values into seven signed 8-bit digits, for products
-// on the FP16 tensor cores that stay as accurate as FP64 (the Ozaki scheme:
+// Split of FP64 values into seven signed 8-bit digits, for products on the FP16
+// tensor cores that are as accurate as FP64 relative to the largest entries that
+// meet (digits, products and sums are exact, the 54-bit operands rounded; the
+// Ozaki scheme:
 // Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
 // multiplication by using fast routines of matrix multiplication and its
 // applications", Numer. Algorithms 59, 2012).
