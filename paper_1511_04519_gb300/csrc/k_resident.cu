@@ -497,28 +497,20 @@ bool res_team(int64_t n, const ResidentPlan& P) {
 }
 }  // namespace
 
-bool resident_set_limits(int64_t n, const ResidentPlan& P) {
-  // the kernels' limits only grow: contexts of several sizes share them
-  static size_t done[2] = {0, 0};
-  const bool team = res_team(n, P);
-  const size_t bytes = team ? res_smem_bytes<WarpTeam>(n, P) : res_smem_bytes<WarpSolo>(n, P);
-  const size_t solve = res_solve_smem_bytes(n, P);
-  bool ok = true;
-  if (bytes > done[team]) {
-    ok = (team ? cudaFuncSetAttribute(resident_round_kernel<WarpTeam>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
-               : cudaFuncSetAttribute(resident_round_kernel<WarpSolo>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) == cudaSuccess;
-    if (ok) done[team] = bytes;
-  }
-  static size_t solve_done = 0;
-  if (ok && solve > solve_done) {
-    ok = cudaFuncSetAttribute(resident_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)solve) == cudaSuccess &&
-         cudaFuncSetAttribute(resident_inputs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)solve) == cudaSuccess;
-    if (ok) solve_done = solve;
-  }
+// The device's own limit for every kernel: nothing to remember between contexts,
+// threads and devices.
+bool resident_set_limits() {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  auto raise = [&](auto kernel) {
+    cudaFuncAttributes a;
+    return cudaFuncGetAttributes(&a, kernel) == cudaSuccess &&
+           cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                optin - (int)a.sharedSizeBytes) == cudaSuccess;
+  };
+  const bool ok = raise(resident_round_kernel<WarpTeam>) && raise(resident_round_kernel<WarpSolo>) &&
+                  raise(resident_solve_kernel) && raise(resident_inputs_kernel);
   if (!ok) cudaGetLastError();
   return ok;
 }

@@ -3,7 +3,6 @@
 #include <cstdint>
 #include <vector>
 #include <cuda_runtime.h>
-#include <cuda_bf16.h>
 
 namespace matex {
 
@@ -485,8 +484,8 @@ void resident_store(const DevFactor& F, const ResStoreSup* sup, int nsup, double
 // whether a grid of n nodes with plan P fits one CTA's shared memory on this
 // device
 bool resident_fits(int64_t n, const ResidentPlan& P);
-// raise the kernels' shared-memory limits for them (false on failure)
-bool resident_set_limits(int64_t n, const ResidentPlan& P);
+// raise the kernels' shared-memory limits to the device's (false on failure)
+bool resident_set_limits();
 // one round: K CTAs, column q of rc by CTA q
 void resident_round(const ResidentArgs& a, int K, cudaStream_t st);
 // the input solves of K columns of rc ahead of their rounds (they depend on

@@ -2930,7 +2930,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
     // resident rounds: one CTA's solve pair and the batched path's
     // single-column pair (in its tuned launch mode), best of five each
     if (plan_resident(c, kResidentThreads) && resident_fits(n, c->rplan) &&
-        resident_set_limits(n, c->rplan)) {
+        resident_set_limits()) {
       c->resident_ok = true;
       cudaMemsetAsync(c->Y, 0, sizeof(double) * (size_t)n * c->ldy, c->st);
       const ResFactor& R1 = o.krylov == 1 ? c->rG : c->rM;
@@ -2987,7 +2987,9 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
   }
   cudaMemsetAsync(c->Vb, 0, sizeof(double) * vslots * kMaxB * n, c->st);
   cudaMemsetAsync(c->Xb, 0, sizeof(double) * G * n, c->st);
-  if (cudaDeviceSynchronize() != cudaSuccess) {
+  // all of it is on c->st; the whole device may not be waited for while another
+  // thread records a run
+  if (cudaStreamSynchronize(c->st) != cudaSuccess) {
     g_setup_err = std::string("setup: ") + cudaGetErrorString(cudaGetLastError());
     delete c;
     return MATEX_ERR_CUDA;
