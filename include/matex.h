@@ -131,9 +131,10 @@ typedef struct matex_opts {
                               tape 0 and tail_eps 0; 2 returns MATEX_ERR_ARG otherwise.  With 0
                               the setup compares them with the batched rounds: by one solve pair
                               each where that decides, else by the time of the context's own
-                              first rounds.  Where the batched rounds win, a run whose new
-                              currents or capacitances change the recorded Krylov dimensions
-                              takes the resident ones (matex_stats.resident of that run).  The
+                              first rounds.  Where the batched rounds win, the first run and
+                              runs whose new currents or capacitances change the recorded
+                              Krylov dimensions take the resident ones all the same (the
+                              matex_stats.resident of that run).  The
                               input solutions of every segment (sources only) are solved ahead
                               of the rounds in one launch when they fit a quarter of the free
                               memory; 3: as 2, but each round kernel solves its own (the path

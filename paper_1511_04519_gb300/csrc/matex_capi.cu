@@ -100,7 +100,7 @@ struct matex_ctx {
   // batched rounds chosen where resident ones fit too: runs with new currents or
   // capacitances may take those (run_device)
   bool res_new = false;      // they may
-  bool new_inputs = false;   // some were set since the last run
+  bool new_inputs = false;   // some were set since the last run (or setup)
   bool drifts = false;       // new ones have changed the recorded counts before
   // resident rounds: every column record's z' and w, solved ahead of the
   // rounds in one launch per run (null: each round kernel solves its own)
@@ -1990,13 +1990,14 @@ matex_status run_resident_once(matex_ctx* c, double* x_out, double t0, matex_sta
 matex_status run_device(matex_ctx* c, double* x_out, matex_stats* stats) {
   const double t0 = now_ms();
   matex_status s;
-  // New inputs mostly change some column's Krylov dimension: the replay is
-  // then lost, and a plain run (the host reads every count) with a new recording
-  // takes two to three replays' time.  Where the resident rounds fit, which hold
-  // no counts, they serve that run, and from then on every run with new inputs.
+  // A plain run (the host reads every count) with its recording takes two to five
+  // replays' time, and pays when the same inputs run again.  Where the resident
+  // rounds fit, which hold no counts, they serve a context's first run; a run
+  // with new inputs whose replay is lost, as they mostly change some column's
+  // Krylov dimension; and from then on every run with new inputs.
   const bool fresh = c->new_inputs && c->res_new && graph_allowed(c);
   c->new_inputs = false;
-  if (fresh && c->drifts) return run_resident_once(c, x_out, t0, stats);
+  if (fresh && (c->drifts || !c->gexec)) return run_resident_once(c, x_out, t0, stats);
   if (graph_allowed(c) && c->gexec) {
     if (cudaGraphLaunch(c->gexec, c->st) != cudaSuccess) return cuda_check(c, "graph launch");
     permute_out(x_out, c->Xp, c->out_map, c->nrows_out, c->n, c->n_times, c->st);
@@ -2964,7 +2965,7 @@ matex_status matex_setup(matex_ctx** out, int64_t n, const double* cap, const in
             c->alloc(c->pre_w, (size_t)c->n_records * n)))
         c->pre_zp = c->pre_w = nullptr;
       c->resident = c->res_pair_ms > 0.f && (o.resident >= 2 || choose_resident(c));
-      c->res_new = c->res_pair_ms > 0.f && !c->resident;
+      c->res_new = c->new_inputs = c->res_pair_ms > 0.f && !c->resident;
     }
     cudaGetLastError();
   }
