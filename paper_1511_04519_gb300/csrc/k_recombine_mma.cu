@@ -5,7 +5,7 @@
 //              V_q y_q(o) + (z_q - w_q) + (t_o - l_q) z'_q            (Eq. 6),
 // as one contraction over k: a column's m basis vectors with the coefficients
 // y_q(o), z'_q with t_o - l_q and z_q - w_q with 1, each zero where the column
-// does not hold o.  Digit products of a 54-bit split (split8.cuh) on
+// does not hold o.  Digit products of a 55-bit split (split8.cuh) on
 // mma.sync: 16 outputs x 8 nodes over 16 terms take the FP64 pipe 1,024 clocks
 // of an SM, the 34 digit products 68.
 //
@@ -158,7 +158,7 @@ rm_coef_kernel(const RmK* __restrict__ list, int ksteps, const double* __restric
   __syncthreads();
   if (threadIdx.x < 16)  // the chunk's exponents; 0x7fff: an inf or NaN among them
     exps[((size_t)blockIdx.x * gridDim.y + blockIdx.y) * 16 + threadIdx.x] =
-        key[threadIdx.x] >= 0x7ff00000 ? 0x7fff : (int16_t)key_exp(key[threadIdx.x]);
+        key[threadIdx.x] >= kKeyInf ? 0x7fff : (int16_t)key_exp(key[threadIdx.x]);
   if (!live) return;
   uint32_t lo[2][kDigits], hi[2][kDigits];
 #pragma unroll
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kRmThreads, 2) rm_gemm_kernel(const __grid_con
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int key = exp_key(v[u]);
-      m = max(m, key >= 0x7ff00000 ? kNonFinite : key_exp(key) - sc[u]);
+      m = max(m, key >= kKeyInf ? kNonFinite : key_exp(key) - sc[u]);
     }
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));

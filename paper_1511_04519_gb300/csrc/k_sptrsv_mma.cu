@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(W * 32, W > 4 ? 2 : 4) mm_level_kernel(const M
         for (int h = 0; h < 2; ++h) {
           if (h && !upper) break;
           const int key = cmax[un.z & 0xffff][g + 8 * h];
-          const int ec = key >= 0x7ff00000 ? kNonFinite : key_exp(key);
+          const int ec = key >= kKeyInf ? kNonFinite : key_exp(key);
 #pragma unroll
           for (int j = 0; j < 2; ++j)
             x[h][j] = few ? compose<true>(c[2 * h + j], er[j] + ec) : compose<false>(c[2 * h + j], er[j] + ec);

@@ -1,4 +1,4 @@
-"""What the digits of the tensor-core solves keep: 54 bits below the largest entry of
+"""What the digits of the tensor-core solves keep: 55 bits below the largest entry of
 a panel row and of a right-hand side over 128 terms.  A solution is then accurate
 relative to its largest entry, on responses that fall over 8 to 50 decades as on
 flat ones: each of about 15 levels is off by at most 128 terms of 2^-54 of the
