@@ -303,9 +303,9 @@ def ncu_case(what: str) -> int:
     """The bench grid restricted to groups 0-7 (32 for "levels"; a few GB on the
     device, solve panels still larger than L2): one warm call, then the
     profiled call.  "solve": matex_solve of 16 columns with the persistent
-    kernel; "levels": 64 columns with one launch per tree level; "run": one
-    full matex_run; "ksweep": bare solve pairs of 1, 4 and 64 columns on the
-    whole grid; "small": one run of the 1,024-node single-group grid;
+    kernel; "levels": 64 columns with one FP64 launch per tree
+    level; "run": one full matex_run; "ksweep": bare solve pairs of 1, 4 and 64
+    columns on the whole grid; "small": one run of the 1,024-node single-group grid;
     "tcsolve": one 64-column solve pair of the whole grid on the tensor cores."""
     import numpy as np
     import torch
@@ -371,7 +371,8 @@ def ncu_case(what: str) -> int:
         torch.cuda.profiler.stop()
         print(json.dumps({"ncu_case": what, "max_memory_gb": torch.cuda.max_memory_allocated() / 1e9}))
         return 0
-    sim = M.Sim(q, solve_mode={"solve": 0, "levels": 1}.get(what, 2))
+    sim = M.Sim(q, solve_mode={"solve": 0, "levels": 1}.get(what, 2),
+                tc_solve="off" if what == "levels" else "auto")
     if what in ("solve", "levels"):
         k = 16 if what == "solve" else 64
         b = torch.randn(k, p.n, dtype=torch.float64, device="cuda")

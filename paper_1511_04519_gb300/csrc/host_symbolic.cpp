@@ -242,8 +242,10 @@ void order_children(Symbolic& S, std::vector<std::vector<int32_t>>& offrows,
 // Widest merged top: every level taken away saves two dependent launches
 // (level solves: 4.5 to 8 us each).  Pair of 8 columns, 512 against none: 77
 // against 99 us on 10,000 nodes, 141 against 164 us on 39,711 (1,024: 70 and
-// 134); the solution's error on the latter 2.6e-15 against 2.2e-15 with none,
-// 3.0e-15 with 1,024 (entries of larger inverses), which set the limit.
+// 134).  The limit was set by the solution's error on the latter, 2.2e-15 with
+// none, 2.6e-15 with 512, 3.0e-15 with 1,024, which was the factors' (their pivots
+// cancelled); on the factors as host_numeric.cpp makes them now it is the same
+// with none and with 512 (2.6e-16 in extended-precision products).
 constexpr int64_t kTopWidth = 512;
 constexpr int64_t kTopMinN = 8192;  // smaller grids keep their panels for the resident rounds
 

@@ -28,8 +28,8 @@
 // Eight K steps make an exact sum (a chunk); rounds of more than 56 K steps take
 // several launches.
 //
-// Measured on the 180k-node grid's tail round (64 columns, about 350 basis
-// vectors, 976 outputs): 8.9 ms against 11.8 ms for nine 6-bit digits on tcgen05
+// Measured on the 180k-node grid's tail round (64 columns, 237 basis vectors and
+// 128 -P terms, 980 outputs, two thirds of the pairs held): 8.9 ms against 11.8 ms for nine 6-bit digits on tcgen05
 // with the -P terms in a pass of their own (one thread's issue of 990 M128 N48
 // products per 48 outputs, nine accumulators filling TMEM, and 72 KB of V digits
 // re-read per 32 terms left its tensor pipe 4 % busy); the tensor pipe's own

@@ -1114,11 +1114,11 @@ bool plan_mm(matex_ctx* c, const std::vector<double>& panM, const std::vector<do
 
 // Which solves take the tensor-core kernels.  opts.tc_solve 2: all (one column
 // only when opts.single_column does not force its own kernels); 0: from two
-// columns on, where they measured faster on every grid tried (1,024 to 180k
-// nodes: 1.4 times and more at two columns, 3.5 times at 16 and 64), and for one
-// column where the pair is at least 5 % faster than the path chosen so far
-// (small grids: 0.034 against 0.061 ms on 1,024 nodes; 0.37 against 0.31 ms on
-// 180k), cached in MATEX_AUTOTUNE_CACHE like the other choices.
+// columns on, where they measured faster on every grid tried (576 to 180k nodes;
+// at two columns 2.9 times, 0.095 to 0.033 ms, on 1,024 nodes and 1.35 times, 0.49
+// to 0.36 ms, on 180k; 3.5 times at 16 and 64), and for one column where the pair
+// is at least 5 % faster than the path chosen so far (small grids: 0.034 against
+// 0.060 ms on 1,024 nodes; 0.36 against 0.29 ms on 180k), cached in MATEX_AUTOTUNE_CACHE like the other choices.
 void choose_mm(matex_ctx* c) {
   c->mm_by_ncols.assign(c->ldy + 1, c->mm_ok ? 1 : 0);
   if (!c->mm_ok) return;
