@@ -15,9 +15,9 @@
 //     node's digits then start at the largest that any column has there, and an
 //     output's at the columns' relative size at that time.  The error is below
 //     2^-54 a term of the first times the second, so that small currents keep
-//     their digits beside large ones and a long tail its own (with the bare
-//     vectors, currents of 1e-12 of the largest lost half of their digits at the
-//     nodes where they act);
+//     their digits beside large ones and a long tail its own (currents of 1e-12
+//     of the largest, at the nodes where they act: off by 2.5e-12 of the terms
+//     with the bare vectors' digits, by less than 1e-13 with these);
 //   rm_coef: per tile of 16 outputs the digits of the K steps that it meets,
 //     and the set of those (a 64-bit mask);
 //   rm_gemm: a CTA splits the vectors' values at its 32 nodes once, keeps the
@@ -29,11 +29,12 @@
 // several launches.
 //
 // Measured on the 180k-node grid's tail round (64 columns, 237 basis vectors and
-// 128 -P terms, 980 outputs, two thirds of the pairs held): 8.9 ms against 11.8 ms for nine 6-bit digits on tcgen05
-// with the -P terms in a pass of their own (one thread's issue of 990 M128 N48
-// products per 48 outputs, nine accumulators filling TMEM, and 72 KB of V digits
-// re-read per 32 terms left its tensor pipe 4 % busy); the tensor pipe's own
-// time is 5.6 ms.  Coefficients as bytes, widened by every warp: 10.1 ms.
+// 128 -P terms, 980 outputs, two thirds of the pairs held): 8.9 ms against 11.8 ms
+// for nine 6-bit digits on tcgen05 with the -P terms in a pass of their own (one
+// thread's issue of 990 M128 N48 products per 48 outputs, nine accumulators
+// filling TMEM, and 72 KB of V digits re-read per 32 terms left its tensor pipe
+// 4 % busy); the tensor pipe's own time is 5.6 ms.  Coefficients as bytes,
+// widened by every warp: 10.1 ms.
 #include <algorithm>
 
 #include "kernels.h"
